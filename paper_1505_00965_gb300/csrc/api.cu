@@ -336,6 +336,31 @@ double problem_cost(int level, int M, const mlmc_payoff *payoff)
     return level_cost(level, M);
 }
 
+// The fixed-point step constants of FP64 paths (level_kernel.cuh, fx_steps).  With |d| <= dmax for
+// every fine step and every normal of the stream (|z| < 7, as above), the running products of a
+// Philox block's four factors satisfy |G - 1| <= (1 + dmax)^4 - 1 < 2^e, and the sum of a coarse
+// step's M increments is at most M dmax < 2^e: the unit is 2^-(63 - e).  e above 3 (dmax above 0.73:
+// sigma sqrt(h) above 0.1) would leave less than FP64's precision; such steps run in FP64.
+static void fill_fixed_point(LevelParams &p, const mlmc_model *m, int M)
+{
+    constexpr double kNormalBound = 7.0;
+    constexpr int kMaxExponent = 3;
+    const bool mil = m->scheme == MLMC_MILSTEIN;
+    const double c2 = 0.5 * m->sigma * m->sigma * p.h, drift = mil ? p.rh - c2 : p.rh;
+    const double dmax = std::fabs(drift) + kNormalBound * p.a + (mil ? kNormalBound * kNormalBound * c2 : 0.0);
+    const double most = std::max(std::pow(1.0 + dmax, 4.0) - 1.0, (double)M * dmax);
+    p.fx = 0;
+    p.fx_a = p.fx_c2 = 0;
+    p.fx_rh = 0;
+    if (m->kind != MLMC_MODEL_GBM || !(most < 0.999 * (1 << kMaxExponent)) || (mil && M > 4)) return;
+    int e = 0;
+    while (!(most < 0.999 * (1 << e))) ++e;
+    p.fx = 63 - e;
+    p.fx_a = (uint64_t)std::nearbyint(std::ldexp(p.a, p.fx + 6));
+    p.fx_c2 = (uint64_t)std::nearbyint(std::ldexp(c2, p.fx + 6));
+    p.fx_rh = (int64_t)std::nearbyint(std::ldexp(drift, p.fx));
+}
+
 void fill_params(LevelParams &p, int level, int M, uint64_t N, uint64_t first,
                  const mlmc_model *m, const mlmc_payoff *pay, uint64_t seed, int tag, int lanes, int precision)
 {
@@ -360,6 +385,9 @@ void fill_params(LevelParams &p, int level, int M, uint64_t N, uint64_t first,
     p.pay_bf = (float)(0.5 * dS0 * p.inv_nf - dK);
     p.pay_ac = (float)(dS0 * p.inv_nc);
     p.pay_bc = (float)(0.5 * dS0 * p.inv_nc - dK);
+    p.pay_dS0_64 = dS0;
+    p.pay_k64 = p.K / p.S0;
+    fill_fixed_point(p, m, M);
     p.first = first;
     p.N = N;
     p.key0 = (uint32_t)seed;

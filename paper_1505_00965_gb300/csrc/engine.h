@@ -23,6 +23,13 @@ struct LevelParams {
     // FP32 payoff constants of the call options on paths relative to S0 (rel_payoff): disc S0,
     // -disc K, and for the fine (f) and coarse (c) path disc S0 / n, disc S0 / (2 n) - disc K
     float pay_dS0, pay_mdK, pay_af, pay_bf, pay_ac, pay_bc;
+    // FP64 payoff constants of the same options: disc S0 and K / S0
+    double pay_dS0_64, pay_k64;
+    // FP64 steps in fixed point (fx_steps): their unit is 2^-fx, 0 where they run in FP64; sigma sqrt(h)
+    // and sigma^2 h / 2 in units of 2^-(fx + 6), r h (Milstein: r h - sigma^2 h / 2) in units of 2^-fx
+    uint64_t fx_a, fx_c2;
+    int64_t fx_rh;
+    int fx;
     uint64_t first;   // first sample index
     uint64_t N;       // number of samples
     uint32_t key0, key1;  // Philox key (seed low, seed high)

@@ -38,6 +38,7 @@ __device__ __forceinline__ void quintic_paths(R x[NS], R h, int n)
 template <typename R, bool TAMED>
 __global__ void __launch_bounds__(256) quintic_level_kernel(const LevelParams p)
 {
+    if constexpr (sizeof(R) == 8) fx_load_tables();
     double m[4] = {0.0, 0.0, 0.0, 0.0};
     float b1 = 0.f, b2 = 0.f, b3 = 0.f, b4 = 0.f;
     int nb = 0;
@@ -51,16 +52,10 @@ __global__ void __launch_bounds__(256) quintic_level_kernel(const LevelParams p)
     for (uint64_t u = t; u < nq; u += T) {
         const uint64_t q = q0 + u;
         const uint4 w = philox4x32_10(make_uint4(p.ctr3, 0u, (uint32_t)(q >> 32), (uint32_t)q), p.rkey);
-        R rho, c, s, x0[4];
-        BoxMuller<R>::pair(w.x, w.y, rho, c, s, u23);
-        x0[0] = rho * c;
-        x0[1] = rho * s;
-        BoxMuller<R>::pair(w.z, w.w, rho, c, s, u23);
-        x0[2] = rho * c;
-        x0[3] = rho * s;
-        R xf[4], xc[4];
+        R x0[4], xf[4], xc[4];
+        block_normals<R>(w, u23, x0);
 #pragma unroll
-        for (int r = 0; r < 4; ++r) xf[r] = xc[r] = x0[r];
+        for (int r = 0; r < 4; ++r) xf[r] = xc[r] = sizeof(R) == 8 ? x0[r] * R(kFxZ) : x0[r];
         quintic_paths<R, TAMED, 4>(xf, h, nf);
         if (coupled) quintic_paths<R, TAMED, 4>(xc, H, nc);
 #pragma unroll
