@@ -479,6 +479,7 @@ int acquire_scratch(size_t ws_bytes, DriverScratch **out)
 {
     int dev = 0;
     CUDA_TRY(cudaGetDevice(&dev));
+    ws_bytes = std::max(ws_bytes, kMinScratchBytes);
     {
         std::lock_guard<std::mutex> lock(g_pool_mutex);
         for (size_t i = 0; i < g_pool.size(); ++i) {
@@ -684,23 +685,24 @@ int mlmc_level_sums_ex(int level, int M, uint64_t N, uint64_t first, const mlmc_
     if (rc) return rc;
     double out[4] = {0.0, 0.0, 0.0, 0.0};
     if (N > 0) {
-        const size_t ws_bytes = workspace_bytes_for_blocks(plan.blocks) + 64;
-        void *ws = nullptr;
-        CUDA_TRY(cudaMallocAsync(&ws, ws_bytes, st));
-        cudaError_t e = cudaMemsetAsync(ws, 0, ws_bytes, st);
+        // buffers from the pool (a stream-ordered allocation costs this call 150 us: the default
+        // pool gives its memory back at every synchronisation); the last block of the kernel
+        // writes the sums to the set's pinned memory
+        DriverScratch *sc = nullptr;
+        rc = acquire_scratch(workspace_bytes_for_blocks(plan.blocks), &sc);
+        if (rc) return rc;
         LevelParams p;
         fill_params(p, level, M, N, first, model, payoff, seed, tag, plan.lanes, precision);
-        p.out = (double *)((char *)ws + workspace_bytes_for_blocks(plan.blocks));
-        if (e == cudaSuccess) rc = launch_level(plan, p, ws, st);
-        else rc = fail(MLMC_ECUDA, "cudaMemsetAsync failed: %s", cudaGetErrorString(e));
-        if (!rc) {
-            e = cudaMemcpyAsync(out, p.out, sizeof(out), cudaMemcpyDeviceToHost, st);
-            if (e != cudaSuccess) rc = fail(MLMC_ECUDA, "cudaMemcpyAsync failed: %s", cudaGetErrorString(e));
-        }
-        cudaFreeAsync(ws, st);
-        e = cudaStreamSynchronize(st);
+        p.out = sc->h_sums;
+        rc = launch_level(plan, p, sc->ws, st);
+        const cudaError_t e = cudaStreamSynchronize(st);
         if (!rc && e != cudaSuccess) rc = fail(MLMC_ECUDA, "level kernel failed: %s", cudaGetErrorString(e));
-        if (rc) return rc;
+        if (rc) {
+            free_scratch(sc);
+            return rc;
+        }
+        std::memcpy(out, sc->h_sums, sizeof(out));
+        release_scratch(sc);
     }
     std::memcpy(sums, out, sizeof(out));
     *cost = (double)N * problem_cost(level, M, payoff);
@@ -775,7 +777,7 @@ extern "C" int mlmc_estimate(double eps, int M, int Lmin, int Lmax, uint64_t N0,
     DriverScratch *sc = nullptr;
     rc = acquire_scratch(ws_slot * kDriverStreams, &sc);
     if (rc) return rc;
-    double *d_sums = sc->d_sums, *h_sums = sc->h_sums;
+    double *h_sums = sc->h_sums;  // pinned: each launch's last block writes its level's sums there
     cudaEvent_t ev0 = sc->ev0, ev1 = sc->ev1;
     RoundStreams rs(sc, st, ws_slot);
     auto cleanup = [&]() { release_scratch(sc); };
@@ -810,7 +812,7 @@ extern "C" int mlmc_estimate(double eps, int M, int Lmin, int Lmax, uint64_t N0,
             LevelParams p;
             fill_params(p, l, M, dN[l], drv.samples_taken(l), model, payoff, seed, MLMC_TAG_PATHS, plan.lanes,
                         precision);
-            p.out = d_sums + 4 * l;
+            p.out = h_sums + 4 * l;
             const int k = rs.take();
             rc = launch_level(plan, p, rs.slot[k], rs.stream[k]);
             if (rc) {
@@ -821,9 +823,8 @@ extern "C" int mlmc_estimate(double eps, int M, int Lmin, int Lmax, uint64_t N0,
         }
         if ((e = rs.join(sc)) != cudaSuccess) return cuda_fail(e, "join of the round's streams");
         if ((e = cudaEventRecord(ev1, st)) != cudaSuccess) return cuda_fail(e, "cudaEventRecord");
-        e = cudaMemcpyAsync(h_sums, d_sums, (L + 1) * 4 * sizeof(double), cudaMemcpyDeviceToHost, st);
         d2h_bytes += (L + 1) * 4 * sizeof(double);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+        e = cudaStreamSynchronize(st);
         if (e != cudaSuccess) return cuda_fail(e, "level round");
         float ms = 0.f;
         if (cudaEventElapsedTime(&ms, ev0, ev1) == cudaSuccess) kernel_ms += ms;

@@ -169,16 +169,18 @@ uint64_t mean_replicates(double kappa, uint64_t dN, uint64_t have)
     return dR;
 }
 
-// Run `body(ws)` with a zeroed stream-ordered workspace of `bytes`, then synchronise.
+// Run `body(ws)` with a workspace of at least `bytes` from the pool (zero ticket, which body's kernels
+// leave zero), then synchronise.
 template <class F> int with_workspace(size_t bytes, cudaStream_t st, F body)
 {
-    void *ws = nullptr;
-    CUDA_TRY(cudaMallocAsync(&ws, bytes, st));
-    cudaError_t e = cudaMemsetAsync(ws, 0, bytes, st);
-    int rc = e == cudaSuccess ? body(ws) : fail(MLMC_ECUDA, "cudaMemsetAsync failed: %s", cudaGetErrorString(e));
-    cudaFreeAsync(ws, st);
-    e = cudaStreamSynchronize(st);
+    DriverScratch *sc = nullptr;
+    int rc = acquire_scratch(bytes, &sc);
+    if (rc) return rc;
+    rc = body(sc->ws);
+    const cudaError_t e = cudaStreamSynchronize(st);
     if (!rc && e != cudaSuccess) rc = fail(MLMC_ECUDA, "control-variate kernel failed: %s", cudaGetErrorString(e));
+    if (rc) free_scratch(sc);
+    else release_scratch(sc);
     return rc;
 }
 
@@ -410,17 +412,13 @@ int mlmc_mlp_forward(const float *params, const float *d_X, uint64_t N, float *d
     int blocks = 0;
     int rc = grid_for((const void *)mlp_forward_kernel, N, &blocks);
     if (rc) return rc;
-    float *d_params = nullptr;
-    CUDA_TRY(cudaMallocAsync(&d_params, sizeof(float) * kNumParams, st));
-    cudaError_t e = cudaMemcpyAsync(d_params, params, sizeof(float) * kNumParams, cudaMemcpyHostToDevice, st);
-    const float *cp = d_params;
-    void *args[] = {(void *)&cp, (void *)&d_X, &N, &d_G};
-    if (e == cudaSuccess) e = cudaLaunchKernel((const void *)mlp_forward_kernel, dim3(blocks), dim3(kCvThreads), args, 0, st);
-    cudaFreeAsync(d_params, st);
-    cudaError_t e2 = cudaStreamSynchronize(st);
-    if (e != cudaSuccess || e2 != cudaSuccess)
-        return fail(MLMC_ECUDA, "network forward failed: %s", cudaGetErrorString(e != cudaSuccess ? e : e2));
-    return MLMC_OK;
+    return with_workspace(kTicketBytes + sizeof(float) * kNumParams, st, [&](void *ws) -> int {
+        const float *d_params = (const float *)((char *)ws + kTicketBytes);
+        CUDA_TRY(cudaMemcpyAsync((void *)d_params, params, sizeof(float) * kNumParams, cudaMemcpyHostToDevice, st));
+        void *args[] = {(void *)&d_params, (void *)&d_X, &N, &d_G};
+        CUDA_TRY(cudaLaunchKernel((const void *)mlp_forward_kernel, dim3(blocks), dim3(kCvThreads), args, 0, st));
+        return MLMC_OK;
+    });
 }
 
 int mlmc_mlp_grad(const float *params, const float *d_X, const float *d_Y, uint64_t N, float *grad, double *loss,

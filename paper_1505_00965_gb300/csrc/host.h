@@ -66,14 +66,17 @@ struct TunedShape {
 };
 bool tuned_lookup(int precision, int payoff, int M, int level, uint64_t N, TunedShape *out);
 
-// Buffers of one adaptive-driver call, pooled per device between calls: a workspace of at least
-// ws_bytes (zero tickets), device and pinned host sums (kDriverSumsPerLevel doubles per level),
+// Buffers of one call with host results (adaptive drivers, level sums, control variate), pooled per
+// device between calls: a workspace of at least ws_bytes (every slot's ticket zero in a set that is
+// in the pool), device and pinned host sums (kDriverSumsPerLevel doubles per level),
 // two timing events, and kDriverStreams - 1 streams with their fork and join events, over which
 // (with the caller's stream) a round spreads its level launches.  acquire_scratch takes a set
 // from the pool or makes one; release_scratch returns it; free_scratch destroys a set that met
 // a CUDA error.
 constexpr int kDriverSumsPerLevel = 16;
 constexpr int kDriverStreams = 4;
+// Every set's workspace holds at least this much, so that the small calls and the drivers share sets.
+constexpr size_t kMinScratchBytes = size_t(1) << 20;
 struct DriverScratch {
     int device = -1;
     void *ws = nullptr;
