@@ -169,7 +169,7 @@ int mlmc_level_sums(int level, int M, uint64_t N, const mlmc_model *model,
  * precision, random-stream tag, launch shape (NULL = automatic) and stream.  Adaptive drivers
  * pass first = the number of samples already taken on this level, so that every round draws
  * new samples.  Host outputs as in mlmc_level_sums; synchronises `stream`.  The engine
- * allocates its small reduction workspace with stream-ordered allocation on `stream`.
+ * takes its small reduction workspace from a pool that mlmc_shutdown releases.
  * Errors: as mlmc_level_sums; MLMC_EINVAL also if first + N overflows 64 bits or the launch
  * shape is invalid for this level.
  */

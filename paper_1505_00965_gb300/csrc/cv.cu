@@ -33,6 +33,7 @@ namespace {
 
 static_assert(kNumParams == MLMC_CV_PARAMS && kInputs == MLMC_CV_INPUTS, "network shape of the C ABI");
 constexpr int kCvThreads = 256;
+constexpr int kGradMaxClusters = 8, kGradSumBlocks = 64;  // mlmc_mlp_grad
 constexpr double kMinKappa = 1.0 / 64.0, kMaxKappa = 4096.0;  // mean points per path sample
 
 const void *cv_data_kernel_for(int payoff)
@@ -226,15 +227,16 @@ int launch_training(const TrainArgs &args, int jobs, int cluster, bool train, cu
     return MLMC_OK;
 }
 
-// Whether a cluster of `cluster` training CTAs fits on this GPU (the SMs of one GPC must hold it).
-bool training_cluster_fits(int cluster, bool train)
+// Clusters of `cluster` training CTAs that this GPU can hold at once (the SMs of one GPC must hold
+// one); 0 if none.
+int training_clusters(int cluster, bool train)
 {
     const void *k = train ? (const void *)train_cluster_kernel<true> : (const void *)train_cluster_kernel<false>;
     if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(TrainSmem)) != cudaSuccess)
-        return false;
+        return 0;
     if (cluster > 8 && cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
         cudaGetLastError();
-        return false;
+        return 0;
     }
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)cluster);
@@ -250,17 +252,17 @@ bool training_cluster_fits(int cluster, bool train)
     int n = 0;
     if (cudaOccupancyMaxActiveClusters(&n, k, &cfg) != cudaSuccess) {
         cudaGetLastError();
-        return false;
+        return 0;
     }
-    return n >= 1;
+    return n;
 }
 
-// Largest cluster (16, 8, 4 or 2 CTAs; at least `least`) that fits and splits B rows into slices
-// of whole 16-row tiles; 0 if none.
-int training_cluster(int B, int least, bool train)
+// Largest cluster (16 or 8 CTAs) that fits and splits B rows into slices of whole 16-row tiles; 0 if
+// none.
+int training_cluster(int B)
 {
-    for (int c = kTrainMaxCluster; c >= least; c /= 2)
-        if (B % (16 * c) == 0 && training_cluster_fits(c, train)) return c;
+    for (int c = kTrainMaxCluster; c >= kTrainMinClusterAdam; c /= 2)
+        if (B % (16 * c) == 0 && training_clusters(c, true) >= 1) return c;
     return 0;
 }
 
@@ -427,34 +429,46 @@ int mlmc_mlp_grad(const float *params, const float *d_X, const float *d_Y, uint6
     if (!params || !d_X || !d_Y || !grad || !loss) return fail(MLMC_EINVAL, "NULL argument");
     if (N == 0 || N % 32 || N > 65536) return fail(MLMC_EINVAL, "N must be a positive multiple of 32, at most 65536");
     cudaStream_t st = (cudaStream_t)stream;
-    const int cluster = training_cluster((int)N, 2, false);
-    if (!cluster) return fail(MLMC_ECUDA, "no thread-block cluster for the gradient kernel fits this GPU");
-    float *d_buf = nullptr;  // parameters, gradient, then N outputs g
-    CUDA_TRY(cudaMallocAsync(&d_buf, sizeof(float) * (2 * kNumParams + N), st));
-    TrainArgs a = {};
-    a.job[0] = TrainJob{d_X, d_Y, d_buf, 0.f, 1.f};
-    a.B = (int)N;
-    a.steps = 1;
-    a.epochs = 1;
-    a.lr = 0.f;
-    a.grad_out = d_buf + kNumParams;
-    a.g_out = d_buf + 2 * kNumParams;
-    std::vector<float> g(N), y(N);
-    cudaError_t e = cudaMemcpyAsync(d_buf, params, sizeof(float) * kNumParams, cudaMemcpyHostToDevice, st);
-    int rc = e == cudaSuccess ? launch_training(a, 1, cluster, false, st)
-                              : fail(MLMC_ECUDA, "upload failed: %s", cudaGetErrorString(e));
-    if (!rc) {
-        e = cudaMemcpyAsync(grad, a.grad_out, sizeof(float) * kNumParams, cudaMemcpyDeviceToHost, st);
-        if (e == cudaSuccess) e = cudaMemcpyAsync(g.data(), a.g_out, sizeof(float) * N, cudaMemcpyDeviceToHost, st);
-        if (e == cudaSuccess) e = cudaMemcpyAsync(y.data(), d_Y, sizeof(float) * N, cudaMemcpyDeviceToHost, st);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-        if (e != cudaSuccess) rc = fail(MLMC_ECUDA, "network gradient failed: %s", cudaGetErrorString(e));
-    }
-    cudaFreeAsync(d_buf, st);
+    // clusters of 16 CTAs (8 where 16 do not fit), as many as the GPU holds at once and as give every
+    // warp a tile of 16 rows; a call with N = 65536 takes 75 us
+    int cluster = kTrainMaxCluster, most = 0;
+    for (; cluster >= 2 && !(most = training_clusters(cluster, false)); cluster /= 2) {}
+    if (!most) return fail(MLMC_ECUDA, "no thread-block cluster for the gradient kernel fits this GPU");
+    const int tiles = (int)(N / 16);
+    const int clusters = std::max(1, std::min({most, kGradMaxClusters, tiles / (kTrainWarps * cluster)}));
+    // workspace: ticket, block sums, parameters, the clusters' gradients, N outputs, loss and gradient
+    const size_t off_par = kTicketBytes + kGradSumBlocks * sizeof(double);
+    const size_t off_parts = off_par + sizeof(float) * (kNumParams + 1);
+    const size_t off_g = off_parts + sizeof(float) * kNumParams * clusters;
+    const size_t off_out = (off_g + sizeof(float) * N + 255) / 256 * 256;
+    struct Out {
+        double loss;
+        float grad[kNumParams];
+    } host;
+    const int rc = with_workspace(off_out + sizeof(Out), st, [&](void *wsv) -> int {
+        char *ws = (char *)wsv;
+        TrainArgs a = {};
+        a.job[0] = TrainJob{d_X, d_Y, (float *)(ws + off_par), 0.f, 1.f};
+        a.B = (int)N;
+        a.steps = 1;
+        a.epochs = 1;
+        a.grad_out = (float *)(ws + off_parts);
+        a.g_out = (float *)(ws + off_g);
+        CUDA_TRY(cudaMemcpyAsync(ws + off_par, params, sizeof(float) * kNumParams, cudaMemcpyHostToDevice, st));
+        int r = launch_training(a, clusters, cluster, false, st);
+        if (r) return r;
+        const float *parts = a.grad_out, *g = a.g_out;
+        int nc = clusters, n = (int)N;
+        double *partials = (double *)(ws + kTicketBytes), *out = (double *)(ws + off_out);
+        unsigned *ticket = (unsigned *)ws;
+        void *args[] = {(void *)&parts, &nc, (void *)&g, (void *)&d_Y, &n, &partials, &ticket, &out};
+        CUDA_TRY(cudaLaunchKernel((const void *)grad_sum_kernel, dim3(kGradSumBlocks), dim3(kGradSumThreads), args, 0, st));
+        CUDA_TRY(cudaMemcpyAsync(&host, out, sizeof(Out), cudaMemcpyDeviceToHost, st));
+        return MLMC_OK;
+    });
     if (rc) return rc;
-    double acc = 0.0;
-    for (uint64_t i = 0; i < N; ++i) acc += ((double)g[i] - y[i]) * ((double)g[i] - y[i]);
-    *loss = acc / (double)N;
+    *loss = host.loss;
+    std::memcpy(grad, host.grad, sizeof(float) * kNumParams);
     return MLMC_OK;
 }
 
@@ -488,7 +502,7 @@ int mlmc_cv_train(int M, const mlmc_model *model, const mlmc_payoff *payoff, uin
             return fail(MLMC_ECUDA, "training stream: %s", cudaGetErrorString(e0));
         }
     }
-    const int cluster = training_cluster(B, kTrainMinClusterAdam, true);
+    const int cluster = training_cluster(B);
     if (!cluster) {
         cudaStreamDestroy(st);
         mlmc_cv_free(cv);
