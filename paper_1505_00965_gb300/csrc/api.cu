@@ -341,6 +341,7 @@ double problem_cost(int level, int M, const mlmc_payoff *payoff)
 // Philox block's four factors satisfy |G - 1| <= (1 + dmax)^4 - 1 < 2^e, and the sum of a coarse
 // step's M increments is at most M dmax < 2^e: the unit is 2^-(63 - e).  e above 3 (dmax above 0.73:
 // sigma sqrt(h) above 0.1) would leave less than FP64's precision; such steps run in FP64.
+// With |1 - K / S0| added to that bound the payoffs of one-block samples fit as well (fixed_block).
 static void fill_fixed_point(LevelParams &p, const mlmc_model *m, int M)
 {
     constexpr double kNormalBound = 7.0;
@@ -348,17 +349,29 @@ static void fill_fixed_point(LevelParams &p, const mlmc_model *m, int M)
     const bool mil = m->scheme == MLMC_MILSTEIN;
     const double c2 = 0.5 * m->sigma * m->sigma * p.h, drift = mil ? p.rh - c2 : p.rh;
     const double dmax = std::fabs(drift) + kNormalBound * p.a + (mil ? kNormalBound * kNormalBound * c2 : 0.0);
-    const double most = std::max(std::pow(1.0 + dmax, 4.0) - 1.0, (double)M * dmax);
     p.fx = 0;
     p.fx_a = p.fx_c2 = 0;
-    p.fx_rh = 0;
-    if (m->kind != MLMC_MODEL_GBM || !(most < 0.999 * (1 << kMaxExponent)) || (mil && M > 4)) return;
-    int e = 0;
-    while (!(most < 0.999 * (1 << e))) ++e;
+    p.fx_rh = p.fx_base = 0;
+    p.fx_fixed = 0;
+    if (m->kind != MLMC_MODEL_GBM) return;
+    // on level 0 the one increment is added to 1 - K / S0 and not multiplied: more of the range is left
+    const bool level0 = p.nf == 1;
+    const double most = level0 ? dmax + std::fabs(1.0 - p.pay_k64)
+                               : std::max(std::pow(1.0 + dmax, 4.0) - 1.0, (double)M * dmax);
+    const int limit = level0 ? kMaxExponent + 1 : kMaxExponent;
+    if (mil && (level0 || M > 4)) return;
+    int e = 0;  // (sigma sqrt(h) must also fit 64 bits in its own unit)
+    while (e <= limit && !(most < 0.999 * (1 << e) && std::ldexp(p.a, 69 - e) < 0x1p64)) ++e;
+    if (e > limit) return;
     p.fx = 63 - e;
     p.fx_a = (uint64_t)std::nearbyint(std::ldexp(p.a, p.fx + 6));
     p.fx_c2 = (uint64_t)std::nearbyint(std::ldexp(c2, p.fx + 6));
     p.fx_rh = (int64_t)std::nearbyint(std::ldexp(drift, p.fx));
+    // payoffs in the same units: the excess 1 - K / S0 + (G - 1) and its difference must fit
+    if (!mil && (level0 || (M == 4 && p.nf == 4)) && (most + std::fabs(1.0 - p.pay_k64) < 0.999 * (1 << e) || level0)) {
+        p.fx_fixed = 1;
+        p.fx_base = (int64_t)std::nearbyint(std::ldexp(1.0 - p.pay_k64, p.fx));
+    }
 }
 
 void fill_params(LevelParams &p, int level, int M, uint64_t N, uint64_t first,
@@ -387,7 +400,6 @@ void fill_params(LevelParams &p, int level, int M, uint64_t N, uint64_t first,
     p.pay_bc = (float)(0.5 * dS0 * p.inv_nc - dK);
     p.pay_dS0_64 = dS0;
     p.pay_k64 = p.K / p.S0;
-    fill_fixed_point(p, m, M);
     p.first = first;
     p.N = N;
     p.key0 = (uint32_t)seed;
@@ -402,6 +414,7 @@ void fill_params(LevelParams &p, int level, int M, uint64_t N, uint64_t first,
     p.nf = (int)nf;
     p.lanes = lanes;
     p.payoff = pay->kind;
+    fill_fixed_point(p, m, M);
     p.c2 = 0.5 * m->sigma * m->sigma * h;
     p.scheme = m->scheme;
     p.fine_only = pay->estimator == MLMC_SINGLE_LEVEL ? 1 : 0;

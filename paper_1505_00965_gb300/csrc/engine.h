@@ -30,6 +30,10 @@ struct LevelParams {
     uint64_t fx_a, fx_c2;
     int64_t fx_rh;
     int fx;
+    // samples of one Philox block at most (level 0; M^l = 4 with M = 4) whose payoff is formed in the
+    // same units: 1 - K / S0, and whether it fits
+    int64_t fx_base;
+    int fx_fixed;
     uint64_t first;   // first sample index
     uint64_t N;       // number of samples
     uint32_t key0, key1;  // Philox key (seed low, seed high)

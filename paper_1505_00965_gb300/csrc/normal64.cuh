@@ -18,8 +18,10 @@
 //   cos, sin quadrant, 512 angles per quadrant by table, the remaining angle delta < pi/1024 by
 //            its Taylor series and the addition theorems.
 //
-// Absolute error of a normal: below 2^-56 (checked against quadruple precision over the edges of
-// every reduction and 10^8 random words), a quarter of the rounding of an FP64 normal of size 1.
+// Error (against quadruple precision, 3e6 random words and the edges of every reduction): cos and sin
+// 2^-59.6 rms and 2^-57 at most, rho 2^-58.7 rms, 2^-56.8 at most from rho = 1/2 on and 2^-53.7 at
+// most (next to u = 1, where rho itself is below 2^-4).  An FP64 normal of size 1 to 2 rounds by up to
+// 2^-53.
 #pragma once
 #include <cstdint>
 #ifndef __CUDACC__
@@ -36,7 +38,21 @@ namespace mlmcgb {
 #ifdef __CUDACC__
 #define MLMC_FX __device__ __forceinline__
 MLMC_FX uint32_t fx_mulhi(uint32_t a, uint32_t b) { return __umulhi(a, b); }
-MLMC_FX int fx_clz(uint32_t a) { return __clz((int)a); }
+MLMC_FX int32_t fx_mulhi_s(int32_t a, int32_t b) { return __mulhi(a, b); }
+// Left shift that brings the top bit to bit 31 (one instruction); -1 for 0.
+MLMC_FX int fx_norm(uint32_t a)
+{
+    int n;
+    asm("bfind.shiftamt.u32 %0, %1;" : "=r"(n) : "r"(a));
+    return n;
+}
+// a << n, 0 for n beyond 31 (n taken unsigned).
+MLMC_FX uint32_t fx_shl(uint32_t a, int n)
+{
+    uint32_t y;
+    asm("shl.b32 %0, %1, %2;" : "=r"(y) : "r"(a), "r"(n));
+    return y;
+}
 MLMC_FX float fx_rcp(float x)
 {
     float y;
@@ -57,7 +73,9 @@ MLMC_FX uint32_t fx_shr_lo(uint32_t lo, uint32_t hi, int k) { return __funnelshi
 #else
 #define MLMC_FX inline
 MLMC_FX uint32_t fx_mulhi(uint32_t a, uint32_t b) { return (uint32_t)(((uint64_t)a * b) >> 32); }
-MLMC_FX int fx_clz(uint32_t a) { return a ? __builtin_clz(a) : 32; }
+MLMC_FX int32_t fx_mulhi_s(int32_t a, int32_t b) { return (int32_t)(((int64_t)a * b) >> 32); }
+MLMC_FX int fx_norm(uint32_t a) { return a ? __builtin_clz(a) : -1; }
+MLMC_FX uint32_t fx_shl(uint32_t a, int n) { return (uint32_t)n > 31u ? 0u : a << n; }
 MLMC_FX float fx_rcp(float x) { return 1.0f / x; }
 MLMC_FX float fx_rsqrt(float x) { return (float)(1.0 / std::sqrt((double)x)); }
 MLMC_FX uint32_t fx_bits(float x)
@@ -89,61 +107,72 @@ MLMC_FX uint64_t fx_mul64x32(uint64_t a, uint32_t b)
     return fx_wide((uint32_t)(a >> 32), b) + fx_mulhi((uint32_t)a, b);
 }
 
-// sqrt(-2 ln(w 2^-32)) in units of 2^-60, w = y + 1 (w = 0 stands for 2^32: the result is 0).
-MLMC_FX uint64_t fx_radius(uint32_t y, const uint64_t *tab)
+// The uniform of a Philox word x as (w mod 2^32) 2^-32 in (0, 1], w = 0 standing for 2^32: the FP64
+// stream's w = x + 1, or the FP32 path's u = 1 - (x mod 2^23) 2^-23, w = -(x << 9).  One multiply-add
+// with uniform factors.
+MLMC_FX uint32_t fx_word(uint32_t x, bool u23) { return x * (u23 ? 0u - 512u : 1u) + (u23 ? 0u : 1u); }
+
+// sqrt(-2 ln(w 2^-32)) in units of 2^-60 (w = 0 stands for 2^32: the result is 0).
+MLMC_FX uint64_t fx_radius(uint32_t w, const uint64_t *tab)
 {
-    const uint32_t w = y + 1u;
-    const int n = fx_clz(w);
-    const uint32_t m = w << (n & 31);
+    const int n = fx_norm(w);
+    const uint32_t m = fx_shl(w, n) | 0x80000000u;
     // k = 512 c, by a magic-number rounding of 2^41 / m
-    const uint32_t k = fx_bits(fmaf(fx_rcp(fx_float(m)), 0x1p41f, 12582912.0f)) - 0x4B400000u;
+    const uint32_t k = fx_bits(fmaf(fx_rcp(fx_float(m)), 0x1p41f, 12582912.0f)) & 0x7FFu;
     const int32_t s = (int32_t)(m * k);  // m k - 2^41: the multiple of 2^32 drops out
-    const uint64_t A = tab[kFxLn2 + (n & 31)] + tab[kFxLnC + ((k - 512u) & 1023u)];  // units of 2^-59
-    // B = -(s - s^2/2 + s^3/3 - s^4/4 + s^5/5) in units of 2^-71
-    const uint64_t q = (uint64_t)((int64_t)s * s);              // 2^-82, below 2^62
-    const uint32_t s2 = (uint32_t)(q >> 30);                    // 2^-52
-    const uint32_t br = 0x55555555u - (uint32_t)(s >> 11) + fx_mulhi(s2, 819u);  // (1/3 - s/4 + s^2/5) 2^32
-    const int64_t tail = (int64_t)s * (int32_t)fx_mulhi(s2, br);  // 2^-93
-    const int64_t B = (int64_t)(q >> 12) - ((int64_t)s << 30) - (tail >> 22);
-    // close to u = 1 (n = 0, c = 1) the table part is 0 and B alone keeps its extra bits
-    const bool near1 = A == 0;
-    const uint64_t F = near1 ? (uint64_t)B : A + (uint64_t)(B >> 12);
+    // n ln 2 + ln c in units of 2^-59; the entry before n = 0 takes w = 0 (n = -1, k = 1024) to 0
+    const uint64_t A = tab[kFxLn2 + n] + tab[kFxLnC + k];
+    // F = -ln u = A - (s - s^2/2 + s^3/3 - s^4/4 + s^5/5)
+    const uint64_t q = (uint64_t)((int64_t)s * s);              // s^2: 2^-82, below 2^62
+    const uint32_t s2 = (uint32_t)(q >> 32);                    // 2^-50
+    const uint32_t br = 0x55555555u - (uint32_t)(s >> 11) + fx_mulhi(s2, 3277u);  // (1/3 - s/4 + s^2/5) 2^32
+    const int64_t tail = (int64_t)s * (int32_t)fx_mulhi(s2, br);  // 2^-91
+    uint64_t F = (uint64_t)((int64_t)s * -(1 << 18) + (int64_t)A) + (q >> 24) - (uint64_t)(int64_t)(int32_t)(tail >> 32);
+    int extra = 0;
+    // next to u = 1 (n = 0, c = 1; one word in 1024) the table part is 0 and the series alone, in units
+    // of 2^-71, keeps the digits that F loses
+    if (A == 0) {
+        F = (q >> 12) - ((uint64_t)(int64_t)s << 30) - (uint64_t)(tail >> 20);
+        extra = 6;
+    }
     // sqrt(2 F): F normalised to x 2^64 by an even shift, x in [1/4, 1)
-    const int e = fx_clz((uint32_t)(F >> 32)) & 30;
+    const int e = fx_norm((uint32_t)(F >> 32)) & 30;
     const uint32_t xh = fx_shl_hi((uint32_t)F, (uint32_t)(F >> 32), e), xl = (uint32_t)F << e;
-    const uint32_t yr = fx_bits(fminf(fx_rsqrt(fx_float(xh)), 0x1.fffffep-16f));
-    // 1 / sqrt(x) in units of 2^-31, lowered by two units of its last place (2^-22, above the
-    // reciprocal root's error of 2^-22.9) so that p = x y stays below 1
-    const uint32_t yi = (yr << 8) - 0x200u;
-    const uint64_t p = fx_mul64x32(fx_join(xl, xh), yi);        // x y: 2^-63
-    const int64_t r = (int64_t)((uint64_t(1) << 62) - fx_mul64x32(p, yi));  // 1 - p y: 2^-62, |r| < 2^42
-    const int32_t rh = (int32_t)(r >> 11);
-    const uint32_t rr = (uint32_t)(((int64_t)rh * rh) >> 32);   // r^2: 2^-70
-    const uint64_t E = (uint64_t)(r + (int64_t)((3u * (rr >> 2)) >> 8)) << 21;  // r + 3 r^2 / 4: 2^-83
-    const int32_t Eh = (int32_t)(E >> 32), ph = (int32_t)(p >> 32), pl = (int32_t)((uint32_t)p >> 1);
-    const int64_t corr = (int64_t)ph * Eh + (((int64_t)pl * Eh) >> 31) + (int64_t)fx_mulhi((uint32_t)ph, (uint32_t)E);
-    const uint64_t root = p + (uint64_t)(corr >> 20);           // 2^-63
-    const int sh = (e >> 1) + (near1 ? 6 : 0);
-    const uint64_t rho = fx_join(fx_shr_lo((uint32_t)root, (uint32_t)(root >> 32), sh), (uint32_t)(root >> 32) >> sh);
-    return w ? rho : 0;
+    // 1 / sqrt(x) in units of 2^-31: the hardware's, lowered by 2^-22 (above its error of 2^-22.9) ...
+    const uint32_t y0 = (fx_bits(fminf(fx_rsqrt(fx_float(xh)), 0x1.fffffep-16f)) << 8) - 0x200u;
+    // ... and corrected by (1 - x y0^2) / 2: x y0^2 in units of 2^-32, less its whole 2^32, is at most
+    // 1.5 2^-30 too low; six units less keep p = x y below 1
+    const uint64_t xyy = fx_wide(xh, fx_mulhi(y0, y0));
+    const uint32_t y = y0 + (uint32_t)fx_mulhi_s((int32_t)(y0 >> 1),
+                                                 (int32_t)(0u - 6u - fx_shr_lo((uint32_t)xyy, (uint32_t)(xyy >> 32), 30)));
+    const uint64_t p = fx_mul64x32(fx_join(xl, xh), y);         // x y: 2^-63
+    // 1 - p y in units of 2^-62, below 2^-28.4; four units more than the products' roundings keep it
+    // above 0 and stand for the halves that the shifts below drop
+    const uint64_t r = (uint64_t(1) << 62) + 4u - fx_mul64x32(p, y);
+    // sqrt(x) = p (1 + r / 2); the next term, 3 r^2 / 8, is below 2^-58 and 2^-61 on average
+    const uint64_t corr = fx_wide((uint32_t)(p >> 32), fx_shr_lo((uint32_t)r, (uint32_t)(r >> 32), 2));  // 2^-92
+    const uint64_t root = p + (corr >> 29);                     // 2^-63
+    const int sh = (e >> 1) + extra;
+    return fx_join(fx_shr_lo((uint32_t)root, (uint32_t)(root >> 32), sh), (uint32_t)(root >> 32) >> sh);
 }
 
-// |cos| and |sin| of 2 pi (y + 1) 2^-32 reduced to the first quadrant, in units of 2^-62, and the
-// quadrant q: (cos, sin) = (c, s), (-s, c), (-c, -s), (s, -c) for q = 0..3.
-MLMC_FX uint32_t fx_circle(uint32_t y, const uint64_t *tab, uint64_t &c, uint64_t &s)
+// |cos| and |sin| of 2 pi t 2^-32 reduced to the first quadrant, in units of 2^-62; in quadrant
+// q = t >> 30, (cos, sin) = (c, s), (-s, c), (-c, -s), (s, -c) for q = 0..3.
+MLMC_FX void fx_circle(uint32_t t, const uint64_t *tab, uint64_t &c, uint64_t &s)
 {
-    const uint32_t t = y + 1u;
     const uint32_t i = (t >> 21) & 511u;
     const uint64_t C = tab[kFxCos + i], S = tab[kFxCos + 512 - i];
     const uint32_t dt = t << 11;                                // delta = 2 pi dt 2^-43 < pi / 1024
     const uint64_t D = fx_mul64x32(kFxTwoPi60, dt);             // delta: 2^-71
-    const uint64_t U = fx_mul64(fx_wide(dt, dt), kFxTwoPiSq59); // delta^2 / 2: 2^-81
-    const uint32_t Uh = (uint32_t)(U >> 32);                    // 2^-49
-    const uint32_t U2 = fx_mulhi(Uh, Uh);                       // delta^4 / 4: 2^-66
+    const uint32_t Dh = (uint32_t)(D >> 32);
+    const uint32_t dl = fx_mulhi((uint32_t)D, Dh);
+    const uint64_t U = fx_wide(Dh, Dh) + dl + dl;               // delta^2 / 2: 2^-79
+    const uint32_t U1 = fx_shr_lo((uint32_t)U, (uint32_t)(U >> 32), 30);  // 2^-49
+    const uint32_t U2 = fx_mulhi(U1, U1);                       // delta^4 / 4: 2^-66
     // u = 1 - cos delta = U - U^2 / 6, v = sin delta = delta - delta (U / 3 - U^2 / 30): 2^-71
-    const uint64_t u = (U >> 10) - ((uint64_t)fx_mulhi(U2, 0x2AAAAAABu) << 5);
-    const uint32_t g = fx_mulhi(Uh, 0xAAAAAAABu) - fx_mulhi(U2, 2185u);  // 2^-50
-    const uint64_t v = D - (fx_wide((uint32_t)(D >> 32), g) >> 18);
+    const uint64_t u = (uint64_t)((int64_t)(int32_t)fx_mulhi(U2, 0x2AAAAAABu) * -32 + (int64_t)(U >> 8));
+    const uint32_t g = fx_mulhi(U1, 0xAAAAAAABu) - fx_mulhi(U2, 2185u);  // 2^-50
+    const uint64_t v = D - (fx_wide(Dh, g) >> 18);
     const uint32_t Ch = (uint32_t)(C >> 32), Cl = (uint32_t)C, Sh = (uint32_t)(S >> 32), Sl = (uint32_t)S;
     const uint32_t uh = (uint32_t)(u >> 32), ul = (uint32_t)u, vh = (uint32_t)(v >> 32), vl = (uint32_t)v;
     // cos = C - (C u + S v), sin = S + (C v - S u); products in units of 2^-69.  The sum of the cross
@@ -155,40 +184,39 @@ MLMC_FX uint32_t fx_circle(uint32_t y, const uint64_t *tab, uint64_t &c, uint64_
     const uint64_t xm = fx_wide(Sh, ul) + fx_wide(Sl, uh);
     const int64_t ps = (int64_t)((fx_wide(Ch, vh) + (xp >> 32)) - (fx_wide(Sh, uh) + (xm >> 32)));
     s = S + (uint64_t)(ps >> 7);
-    return t >> 30;
 }
-
-// The FP64 stream takes the 32 bits of a word; the FP32 path's stream u = 1 - (x mod 2^23) 2^-23,
-// the same fixed-point uniform (y + 1) 2^-32 with y = ~(x << 9).
-MLMC_FX uint32_t fx_word(uint32_t x, bool u23) { return u23 ? ~(x << 9) : x; }
+// Signs of the cosine and sine of angle t as all-ones masks, and whether they trade places.
+MLMC_FX uint64_t fx_cos_sign(uint32_t t) { return (uint64_t)(int64_t)((int32_t)(t + 0x40000000u) >> 31); }
+MLMC_FX uint64_t fx_sin_sign(uint32_t t) { return (uint64_t)(int64_t)((int32_t)t >> 31); }
+MLMC_FX bool fx_swapped(uint32_t t) { return (t & 0x40000000u) != 0; }
 
 // The two normals of a word pair, in units of 2^-58.
 constexpr double kFxZ = 0x1p-58;
 MLMC_FX void fx_pair(uint32_t xa, uint32_t xb, bool u23, const uint64_t *tab, int64_t &z0, int64_t &z1)
 {
     const uint64_t rho = fx_radius(fx_word(xa, u23), tab);
+    const uint32_t t = fx_word(xb, u23);
     uint64_t c, s;
-    const uint32_t q = fx_circle(fx_word(xb, u23), tab, c, s);
-    const bool swap = q & 1;
-    const uint64_t m0 = (q == 1 || q == 2) ? ~uint64_t(0) : 0, m1 = q >= 2 ? ~uint64_t(0) : 0;
-    z0 = (int64_t)((fx_mul64(rho, swap ? s : c) ^ m0) - m0);
-    z1 = (int64_t)((fx_mul64(rho, swap ? c : s) ^ m1) - m1);
+    fx_circle(t, tab, c, s);
+    const uint64_t m0 = fx_cos_sign(t), m1 = fx_sin_sign(t);
+    z0 = (int64_t)((fx_mul64(rho, fx_swapped(t) ? s : c) ^ m0) - m0);
+    z1 = (int64_t)((fx_mul64(rho, fx_swapped(t) ? c : s) ^ m1) - m1);
 }
 
 // x 2^-unit rounded to FP64 (half up), x at least 2^32; `any` also takes smaller x and 0.
 template <bool any = false> MLMC_FX uint64_t fx_double_bits(uint64_t x, int unit)
 {
     uint32_t hi = (uint32_t)(x >> 32), lo = (uint32_t)x;
-    int n = fx_clz(hi);
+    int top = 1023 + 62 - unit;
     if (any && hi == 0) {
         hi = lo;
         lo = 0;
-        n = 32 + fx_clz(hi);
+        top -= 32;
     }
+    const int n = fx_norm(hi);
     const uint32_t vh = fx_shl_hi(lo, hi, n & 31), vl = lo << (n & 31);
-    const uint64_t r = fx_join(fx_shr_lo(vl, vh, 11), (vh >> 11) + (uint32_t)(1023 + 62 - unit - n) * 0x100000u) +
-                       ((vl >> 10) & 1u);
-    return any && x == 0 ? 0 : r;
+    const uint64_t r = fx_join(fx_shr_lo(vl, vh, 11), (vh >> 11) + (uint32_t)(top - n) * 0x100000u) + ((vl >> 10) & 1u);
+    return any && hi == 0 ? 0 : r;
 }
 
 // The high 64 bits of the signed product a b, within 2 and without a bias: the addend stands for the
@@ -202,18 +230,27 @@ MLMC_FX int64_t fx_mul64s(int64_t a, int64_t b)
     return (int64_t)ah * bh + (cross >> 31);
 }
 
+// Running products G_k = (1 + d_0) .. (1 + d_{k-1}) of four increments as D_k = G_k - 1, all in units of
+// 2^-(64 - up) (fx_mul64s returns units of 2^-(64 - 2 up)).
+MLMC_FX void fx_products(int64_t d0, int64_t d1, int64_t d2, int64_t d3, int up, int64_t &D2, int64_t &D3, int64_t &D4)
+{
+    D2 = d0 + d1 + (int64_t)((uint64_t)fx_mul64s(d0, d1) << up);
+    D3 = D2 + d2 + (int64_t)((uint64_t)fx_mul64s(D2, d2) << up);
+    D4 = D3 + d3 + (int64_t)((uint64_t)fx_mul64s(D3, d3) << up);
+}
+
 // Relative increments d = r h + sigma dW of one word pair's two fine steps in units of 2^-u:
 // A is sigma sqrt(h) in units of 2^-(u + 6), rh is r h in units of 2^-u.
 MLMC_FX void fx_increment_pair(uint32_t xa, uint32_t xb, bool u23, const uint64_t *tab, uint64_t A, int64_t rh,
                                int64_t &d0, int64_t &d1)
 {
     const uint64_t ra = fx_mul64(fx_radius(fx_word(xa, u23), tab), A);
+    const uint32_t t = fx_word(xb, u23);
     uint64_t c, s;
-    const uint32_t q = fx_circle(fx_word(xb, u23), tab, c, s);
-    const bool swap = q & 1;
-    const uint64_t m0 = (q == 1 || q == 2) ? ~uint64_t(0) : 0, m1 = q >= 2 ? ~uint64_t(0) : 0;
-    d0 = rh + (int64_t)((fx_mul64(ra, swap ? s : c) ^ m0) - m0);
-    d1 = rh + (int64_t)((fx_mul64(ra, swap ? c : s) ^ m1) - m1);
+    fx_circle(t, tab, c, s);
+    const uint64_t m0 = fx_cos_sign(t), m1 = fx_sin_sign(t);
+    d0 = rh + (int64_t)((fx_mul64(ra, fx_swapped(t) ? s : c) ^ m0) - m0);
+    d1 = rh + (int64_t)((fx_mul64(ra, fx_swapped(t) ? c : s) ^ m1) - m1);
 }
 // The Milstein increment r h - c2 + sigma sqrt(h) z + c2 z^2 from z in units of 2^-58; A and C2 in
 // units of 2^-(u + 6), rhm in units of 2^-u.
@@ -228,10 +265,13 @@ __device__ __forceinline__ double fx_to_double(uint64_t x, int unit)
 {
     return __longlong_as_double((long long)fx_double_bits(x, unit));
 }
+// The FP64 pipe converts a signed 64-bit integer in one operation, 64 cycles per warp and scheduler
+// against 60 of the integer pipes; the steps keep those busy.
 __device__ __forceinline__ double fx_to_double_signed(int64_t x, int unit)
 {
-    const uint64_t m = (uint64_t)(x >> 63);
-    return __longlong_as_double((long long)(fx_double_bits<true>(((uint64_t)x ^ m) - m, unit) | (m << 63)));
+    const double d = (double)x;
+    const int hi = __double2hiint(d);
+    return __hiloint2double(hi ? hi - (unit << 20) : 0, __double2loint(d));
 }
 // The block's copy of the tables (8.5 KB of shared memory, one instance per kernel), filled by
 // fx_load_tables, which ends with a block barrier.

@@ -21,8 +21,12 @@ using namespace mlmcgb;
 extern "C" void pairs(const uint32_t *y, long n, uint64_t *rho, uint64_t *c, uint64_t *s, uint32_t *q)
 {
     for (long i = 0; i < n; ++i) {
-        rho[i] = fx_radius(y[i], kFxTables);
-        q[i] = fx_circle(y[i], kFxTables, c[i], s[i]);
+        const uint32_t w = fx_word(y[i], false);
+        rho[i] = fx_radius(w, kFxTables);
+        fx_circle(w, kFxTables, c[i], s[i]);
+        const bool minus_c = fx_cos_sign(w) != 0, minus_s = fx_sin_sign(w) != 0;
+        q[i] = fx_swapped(w) ? (minus_c ? 1 : 3) : (minus_c ? 2 : 0);  // and minus_s from quadrant 2 on
+        if (minus_s != (q[i] >= 2)) q[i] = 9;
     }
 }
 extern "C" void doubles(const uint64_t *x, long n, int unit, uint64_t *d)
