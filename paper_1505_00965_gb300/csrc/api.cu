@@ -25,8 +25,6 @@ namespace {
 
 thread_local std::string g_error;
 
-// Least cost of a launch with fewer items than one wave, in waves (see plan_level)
-constexpr double kLoneWaveCost = 0.25;
 // Samples per thread of one-thread-per-sample FP32 launches when neither the caller nor the
 // autotuner chose.
 constexpr int kDefaultSamplesPerThread = 1;
@@ -148,18 +146,14 @@ int plan_level(int level, int M, uint64_t N, int precision, int payoff, int sche
             return fail(MLMC_EINVAL, "lanes_per_path %d does not divide M^l = %ld into chunks of a "
                         "multiple of %d steps", lanes, nf, unit);
     } else {
-        // The power of two P (chunks of whole Philox blocks and coarse steps, at least 256 steps
-        // each) with the least modelled launch time.  T resident threads run the N P lane-items
-        // in waves; after w >= 1 whole waves, a partial last wave filled to a fraction f costs
-        // min(1, 1.25 f + 0.1) of a full one (its warps run faster on the emptier SMs), and a
-        // launch of fewer items than a wave min(1, 3 f).  A lane costs its M^l / P steps plus
-        // about 12 steps of chunk join, payoff and moments, and a split step about 8 % more than
-        // a whole-path one (two samples per thread).  A larger P must win by more than 1 %.
-        // (Fitted to launch timings of the lookback, levels 5..8 at 0.2..3.7 waves: 1.3-1.6 %
-        // less time per level than the earlier fit.)  Fewer items than one wave still cost at least a
-        // quarter of a wave: a warp alone on its scheduler takes about 64 cycles per step,
-        // against about 266 for each warp of a full SM (measured on levels 6..12 at 1 to 2^15
-        // samples), so short launches go to the most lanes.
+        // The power of two P (chunks of whole Philox blocks and coarse steps, at least min_lane_steps
+        // steps each) with the least modelled launch time.  T resident threads run the N P lane-items
+        // in waves (lane_waves).  A lane costs its M^l / P steps plus about 12 steps of chunk join,
+        // payoff and moments, and a split step about 8 % more than a whole-path one (two samples per
+        // thread).  A larger P must win by more than 1 %.  (FP32: fitted to launch timings of the
+        // lookback, levels 5..8 at 0.2..3.7 waves; a warp alone on its scheduler takes about 64 cycles
+        // per step, against about 266 for each warp of a full SM, measured on levels 6..12 at 1 to
+        // 2^15 samples, so short launches go to the most lanes.)
         lanes = 1;
         if (nf >= 8) {
             const int mt1 = M == 4 ? 4 : 0;
@@ -174,13 +168,11 @@ int plan_level(int level, int M, uint64_t N, int precision, int payoff, int sche
             rc = max_resident_blocks(kp, threads, &resp);
             if (rc) return rc;
             double best = 0.0;
+            const bool fp64 = precision != MLMC_FP32_PATH;
             for (int P = 1; P <= 32; P *= 2) {
-                if (P > 1 && (nf % P != 0 || (nf / P) % unit != 0 || nf / P < 256)) break;
+                if (P > 1 && (nf % P != 0 || (nf / P) % unit != 0 || nf / P < min_lane_steps(fp64))) break;
                 const double T = (double)(P == 1 ? res1 : resp) * threads;
-                const double w = (double)std::max<uint64_t>(N, 1) * P / T;
-                const double full = std::floor(w);
-                const double waves = w < 1.0 ? std::max(std::min(1.0, 3.0 * w), kLoneWaveCost)
-                                             : full + std::min(1.0, kLanesTailSlope * (w - full) + kLanesTailBase);
+                const double waves = lane_waves((double)std::max<uint64_t>(N, 1) * P / T, fp64);
                 const double per_step = P > 1 ? kLanesSplitStep : 1.0;
                 const double cost = waves * ((double)nf / P + 12.0) * per_step;
                 if (P == 1 || cost < 0.99 * best) {
@@ -287,8 +279,31 @@ bool positive_step_factors(const mlmc_model *m, int level, int M)
            1.0 + m->r * H - m->sigma * M * std::sqrt(h) * kNormalBound > kMargin;
 }
 
+// Launches that leave most of the GPU idle (plan: the shape found so far, automatic fields zero in
+// launch).  Blocks shrink to 128 and 64 threads while the grid has fewer blocks than the GPU has SMs;
+// this regroups the FP64 partial sums only (every thread has one sample at most).  A warp that has its
+// scheduler to itself runs a Philox call in about 245 cycles, two on one scheduler in about 305:
+// level 6 with 19,456 samples on whole paths 171 us with 256 threads, 121 with 64.
+static int plan_idle(int level, int M, uint64_t N, int precision, const mlmc_model *model, const mlmc_payoff *payoff,
+                     const mlmc_launch *launch, Plan *plan)
+{
+    const long nf = ipow(M, level);
+    int sms = 0;
+    int rc = device_sms(&sms);
+    if (rc) return rc;
+    TunedShape shape;
+    const bool tuned = model->scheme == MLMC_EULER_MARUYAMA && tuned_lookup(precision, payoff->kind, M, level, N, &shape);
+    if (!tuned && !(launch && (launch->threads_per_block || launch->blocks))) {
+        const double items = nf < 4 ? std::ceil((double)std::max<uint64_t>(N, 1) * nf / 4.0) + 1.0
+                                    : (double)std::max<uint64_t>(N, 1) * plan->lanes;
+        while (plan->threads > 64 && plan->threads % 64 == 0 && std::ceil(items / plan->threads) < sms) plan->threads /= 2;
+        if (plan->threads < 256) plan->blocks = std::max(1, (int)std::ceil(items / plan->threads));
+    }
+    return MLMC_OK;
+}
+
 int plan_problem(int level, int M, uint64_t N, int precision, const mlmc_model *model, const mlmc_payoff *payoff,
-                 const mlmc_launch *launch, Plan *plan)
+                 const mlmc_launch *launch, Plan *plan, bool spread)
 {
     if (model->kind == MLMC_MODEL_QUINTIC_ODE) return plan_ode(level, M, N, precision, model->scheme, launch, plan);
     if (payoff->estimator != MLMC_ANTITHETIC) {
@@ -302,7 +317,7 @@ int plan_problem(int level, int M, uint64_t N, int precision, const mlmc_model *
                                 : level_kernel_fp64(payoff->kind, mt, true, model->scheme, false, true);
             if (k) plan->kernel = k;
         }
-        return MLMC_OK;
+        return spread ? plan_idle(level, M, N, precision, model, payoff, launch, plan) : MLMC_OK;
     }
     // antithetic: one thread per sample; the kernel of levels with M^l < 4 reads the flag
     if (M != 2 && M != 4) return fail(MLMC_ENOTIMPL, "the antithetic estimator is built for M = 2 and 4 (M = %d)", M);
@@ -315,7 +330,8 @@ int plan_problem(int level, int M, uint64_t N, int precision, const mlmc_model *
     one.lanes_per_path = 1;
     one.samples_per_thread = 1;
     int rc = plan_level(level, M, N, precision, payoff->kind, model->scheme, &one, plan);
-    if (rc || ipow(M, level) < 4) return rc;
+    if (rc) return rc;
+    if (ipow(M, level) < 4) return spread ? plan_idle(level, M, N, precision, model, payoff, launch, plan) : MLMC_OK;
     const int mt = M == 4 ? 4 : 0;
     const bool long_lanes = ipow(M, level) > kLongLaneSteps;
     plan->kernel = precision == MLMC_FP32_PATH ? level_anti_kernel_fp32(payoff->kind, mt, model->scheme, long_lanes)
@@ -325,7 +341,7 @@ int plan_problem(int level, int M, uint64_t N, int precision, const mlmc_model *
     rc = max_resident_blocks(plan->kernel, plan->threads, &resident);
     if (rc) return rc;
     if (!(launch && launch->blocks)) plan->blocks = std::max(1, std::min(plan->blocks, resident));
-    return MLMC_OK;
+    return spread ? plan_idle(level, M, N, precision, model, payoff, launch, plan) : MLMC_OK;
 }
 
 double problem_cost(int level, int M, const mlmc_payoff *payoff)
@@ -816,7 +832,7 @@ extern "C" int mlmc_estimate(double eps, int M, int Lmin, int Lmax, uint64_t N0,
         for (int l = L; l >= 0; --l) {
             if (!dN[l]) continue;
             Plan plan;
-            rc = plan_problem(l, M, dN[l], precision, model, payoff, nullptr, &plan);
+            rc = plan_problem(l, M, dN[l], precision, model, payoff, nullptr, &plan, false);
             if (!rc && plan.blocks > ws_blocks) plan.blocks = ws_blocks;
             if (rc) {
                 free_scratch(sc);  // waits for the launches already queued on the set's streams

@@ -1,5 +1,6 @@
 // engine.h -- internal interface between the C ABI and the level kernels.
 #pragma once
+#include <cmath>
 #include <cstddef>
 #include <cstdint>
 
@@ -90,10 +91,23 @@ constexpr int kNs2MaxThreads = 512;
 // on the Asian, 4.5 % over the whole set.  On the straight-line sample of M^l = 4 two samples per
 // thread were slower.
 constexpr long kNs2MinSteps = 16;
-// The lanes-per-path model of both planners (plan_level and the device rounds): the cost of a
-// partial last wave after whole ones, min(1, kLanesTailSlope f + kLanesTailBase) of a wave at
-// fill f, and a split step's cost relative to a whole-path one.
+// The lanes-per-path model of both planners (plan_level and the device rounds): the time of w waves
+// of lane-items in whole waves (a partial last wave after whole ones costs min(1, kLanesTailSlope f
+// + kLanesTailBase) at fill f), a split step's cost relative to a whole-path one, and the least steps
+// of a lane.  Below one wave FP32 paths wait on latency: min(1, 3 w), and a quarter of a wave at
+// least.  FP64 paths, integer arithmetic of four times the instructions per step, fill a scheduler
+// with a few warps: launches of levels 3..7 at 0.02..0.96 waves took 0.26 of a wave up to w = 0.06,
+// then 0.34, 0.56 and 0.82 at w = 0.16, 0.32 and 0.64 (3112 samples: level 4 76 -> 31 us, level 6
+// 0.96 -> 0.12 ms against one lane each).
 constexpr double kLanesTailSlope = 1.25, kLanesTailBase = 0.1, kLanesSplitStep = 1.08;
+__host__ __device__ inline double lane_waves(double w, bool fp64)
+{
+    const double full = floor(w), tail = kLanesTailSlope * (w - full) + kLanesTailBase;
+    if (w >= 1.0) return full + (tail < 1.0 ? tail : 1.0);
+    const double part = fp64 ? 0.2 + 0.95 * w : 3.0 * w, least = fp64 ? 0.26 : 0.25;
+    return part < least ? least : part < 1.0 ? part : 1.0;
+}
+__host__ __device__ constexpr long min_lane_steps(bool fp64) { return fp64 ? 32 : 256; }
 // The control variate's level-estimator kernel (cv_level.cu) for a payoff on level `level` with
 // refinement M: compiled for M^l = 1, 4, 16 at M = 4, else for a run-time M^l; NULL for an unknown
 // payoff.

@@ -38,7 +38,6 @@ constexpr int kGdVariants = 3;  // per level: one thread per path (or the small 
 constexpr int kGdNodes = MLMC_MAX_LEVELS * kGdVariants;
 constexpr int kGdThreads = 256;
 constexpr int kGdMaxIterations = 4096;  // estimates take tens of rounds
-constexpr double kGdLoneWaveCost = 0.25;
 
 enum : int { kGdRunning = 0, kGdDone = 1, kGdNonFinite = 2, kGdDeviceError = 3, kGdTooManyRounds = 4 };
 enum : int { kVarWhole = 0, kVarSplit = 1, kVarSplitLong = 2 };
@@ -56,6 +55,7 @@ struct GdState {
     int M, Lmin, Lmax;
     int small_levels;   // levels l < small_levels have M^l < 4 (4 / M^l samples per Philox block)
     int antithetic;     // one thread per sample, no split
+    int fp64;           // FP64 paths (the lanes model's second fit)
     int ws_blocks;      // grid cap: blocks of a level's workspace slot
     uint64_t N0;
     int res1[MLMC_MAX_LEVELS], resp[MLMC_MAX_LEVELS];  // residencies the lanes model compares
@@ -160,12 +160,9 @@ __device__ void gd_plan(const GdState &s, int l, uint64_t dN, int &variant, int 
         if (nf >= 8 && !s.antithetic) {
             double best = 0.0;
             for (int P = 1; P <= 32; P *= 2) {
-                if (P > 1 && (nf % P != 0 || (nf / P) % unit != 0 || nf / P < 256)) break;
+                if (P > 1 && (nf % P != 0 || (nf / P) % unit != 0 || nf / P < min_lane_steps(s.fp64 != 0))) break;
                 const double T = (double)(P == 1 ? s.res1[l] : s.resp[l]) * threads;
-                const double w = Nd * P / T;
-                const double full = floor(w);
-                const double waves = w < 1.0 ? fmax(fmin(1.0, 3.0 * w), kGdLoneWaveCost)
-                                             : full + fmin(1.0, kLanesTailSlope * (w - full) + kLanesTailBase);
+                const double waves = lane_waves(Nd * P / T, s.fp64 != 0);
                 const double per_step = P > 1 ? kLanesSplitStep : 1.0;
                 const double cost = waves * ((double)nf / P + 12.0) * per_step;
                 if (P == 1 || cost < 0.99 * best) {
@@ -640,6 +637,7 @@ int estimate_on_device(double eps, int M, int Lmin, int Lmax, uint64_t N0, const
     while (small <= Lmax && ipow(M, small) < 4) ++small;
     h.small_levels = small;
     h.antithetic = payoff->estimator == MLMC_ANTITHETIC ? 1 : 0;
+    h.fp64 = precision != MLMC_FP32_PATH ? 1 : 0;
     h.ws_blocks = c->ws_blocks;
     AdaptiveMLMC costs(eps, M, Lmin, Lmax, N0);  // C_l with the estimator's cost scale
     if (h.antithetic)

@@ -48,8 +48,10 @@ int estimate_on_device(double eps, int M, int Lmin, int Lmax, uint64_t N0, const
                        const mlmc_payoff *payoff, uint64_t seed, int precision, cudaStream_t st, mlmc_result *out,
                        std::chrono::steady_clock::time_point t_start);
 void graph_driver_release(int dev);
+// spread: whether launches that leave SMs idle may take smaller blocks (the adaptive driver keeps 256
+// threads, the shape of its device rounds, whose sums its own repeat bit for bit).
 int plan_problem(int level, int M, uint64_t N, int precision, const mlmc_model *model, const mlmc_payoff *payoff,
-                 const mlmc_launch *launch, Plan *plan);
+                 const mlmc_launch *launch, Plan *plan, bool spread = true);
 void fill_params(LevelParams &p, int level, int M, uint64_t N, uint64_t first,
                  const mlmc_model *m, const mlmc_payoff *pay, uint64_t seed, int tag, int lanes, int precision);
 double level_cost(int level, int M);
