@@ -190,6 +190,10 @@ int plan_level(int level, int M, uint64_t N, int precision, int payoff, int sche
     const bool ns2_ok = !split && !small && precision == MLMC_FP32_PATH && scheme == MLMC_EULER_MARUYAMA &&
                         threads <= kNs2MaxThreads;
     const int auto_ns = ns2_ok && M == 4 && nf >= kNs2MinSteps ? 2 : kDefaultSamplesPerThread;
+    // Milstein paths take their two-sample kernel by default only (the field asks for Euler--Maruyama)
+    const void *mil2 = scheme == MLMC_MILSTEIN && !split && !small && !ns_req
+                           ? default_ns2_kernel(precision == MLMC_FP32_PATH, payoff, M, nf, scheme, false, threads)
+                           : nullptr;
     int ns = ns_req ? ns_req : (have_tuned && tuned.ns ? tuned.ns : auto_ns);
     if (ns == 2 && !ns2_ok) {
         if (ns_req == 2)
@@ -197,7 +201,8 @@ int plan_level(int level, int M, uint64_t N, int precision, int payoff, int sche
                         "lanes_per_path 1 and at most %d threads per block", kNs2MaxThreads);
         ns = 1;
     }
-    plan->kernel = ns == 2 ? level_ns2_kernel_fp32(payoff, mt, long_lanes)
+    plan->kernel = ns == 2 ? level_ns2_kernel_fp32(payoff, mt, scheme, false, long_lanes)
+                 : mil2 ? mil2
                  : precision == MLMC_FP32_PATH ? level_kernel_fp32(payoff, mt, split, scheme, long_lanes)
                                                : level_kernel_fp64(payoff, mt, split, scheme, long_lanes);
     if (!plan->kernel) return fail(MLMC_EINVAL, "no kernel for payoff %d", payoff);
@@ -336,6 +341,11 @@ int plan_problem(int level, int M, uint64_t N, int precision, const mlmc_model *
     const bool long_lanes = ipow(M, level) > kLongLaneSteps;
     plan->kernel = precision == MLMC_FP32_PATH ? level_anti_kernel_fp32(payoff->kind, mt, model->scheme, long_lanes)
                                                : level_anti_kernel_fp64(payoff->kind, mt, model->scheme, long_lanes);
+    if (!(launch && launch->samples_per_thread)) {
+        const void *k = default_ns2_kernel(precision == MLMC_FP32_PATH, payoff->kind, M, ipow(M, level), model->scheme, true,
+                                           plan->threads);
+        if (k) plan->kernel = k;
+    }
     if (!plan->kernel) return fail(MLMC_EINVAL, "no antithetic kernel for payoff %d", payoff->kind);
     int resident = 0;
     rc = max_resident_blocks(plan->kernel, plan->threads, &resident);

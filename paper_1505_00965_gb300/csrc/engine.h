@@ -79,18 +79,21 @@ const void *level_kernel_fp64_milstein(int payoff, int mt, bool split, bool long
 // Antithetic level kernels (level_anti_fp32.cu, level_anti_fp64.cu): mt = 4 (M = 4) or 0 (M = 2).
 const void *level_anti_kernel_fp32(int payoff, int mt, int scheme, bool long_lanes);
 const void *level_anti_kernel_fp64(int payoff, int mt, int scheme, bool long_lanes);
-// Two samples per thread (level_fp32_ns2.cu): FP32 paths, Euler--Maruyama, one thread per sample,
-// mt = 4 or 0; at most 512 threads per block.
-const void *level_ns2_kernel_fp32(int payoff, int mt, bool long_lanes);
+// Two samples per thread (level_fp32_ns2.cu, level_fp32_ns2_mil.cu): FP32 paths, one thread per
+// sample, at most 512 threads per block; Euler--Maruyama for mt = 4 or 0, Milstein and the antithetic
+// estimator for mt = 4 (NULL where there is none).
+const void *level_ns2_kernel_fp32(int payoff, int mt, int scheme, bool anti, bool long_lanes);
+const void *level_ns2_kernel_fp32_other(int payoff, int mt, int scheme, bool anti, bool long_lanes);
 constexpr int kNs2MaxThreads = 512;
-// The planners' default of two samples per thread: FP32 Euler--Maruyama whole paths with M = 4
-// and at least 16 fine steps.  The two-sample kernel takes the same samples per thread on the
-// same grid (a thread's unpaired last sample runs alone).  Timed against one sample per thread on
-// the lookback and arithmetic Asian calls at levels 2-7 and 0.3-6.4 waves of resident threads, it
-// was 0.6 % slower in one case of 84 and faster in the rest: about 3 % on the lookback and 3-8 %
-// on the Asian, 4.5 % over the whole set.  On the straight-line sample of M^l = 4 two samples per
-// thread were slower.
+// The planners' default of two samples per thread: FP32 whole paths with M = 4 and at least 16 fine
+// steps.  The two-sample kernel takes the same samples per thread in the same order on the same grid
+// (a thread's unpaired last sample runs alone).
 constexpr long kNs2MinSteps = 16;
+inline const void *default_ns2_kernel(int precision_is_fp32, int payoff, int M, long nf, int scheme, bool anti, int threads)
+{
+    if (!precision_is_fp32 || M != 4 || nf < kNs2MinSteps || threads > kNs2MaxThreads) return nullptr;
+    return level_ns2_kernel_fp32(payoff, 4, scheme, anti, nf > kLongLaneSteps);
+}
 // The lanes-per-path model of both planners (plan_level and the device rounds): the time of w waves
 // of lane-items in whole waves (a partial last wave after whole ones costs min(1, kLanesTailSlope f
 // + kLanesTailBase) at fill f), a split step's cost relative to a whole-path one, and the least steps

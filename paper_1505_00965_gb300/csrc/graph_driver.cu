@@ -416,11 +416,10 @@ int level_kernels(int l, int M, int precision, const mlmc_model *model, const ml
         return max_resident_blocks(out->k[kVarWhole], kGdThreads, &out->resident[kVarWhole]);
     }
     const int mt = M == 4 ? 4 : 0;
-    // whole paths: the two-sample kernel where plan_level takes it by default (same grid rule)
-    const bool ns2 = !anti && precision == MLMC_FP32_PATH && scheme == MLMC_EULER_MARUYAMA && M == 4 &&
-                     nf >= kNs2MinSteps && kGdThreads <= kNs2MaxThreads;
-    const void *whole = ns2 ? level_ns2_kernel_fp32(pay, mt, nf > kLongLaneSteps)
-                            : pick(mt, false, nf > kLongLaneSteps, false);
+    // whole paths: the two-sample kernel where plan_level takes it by default (same grid rule; the
+    // antithetic estimator's own follows below)
+    const void *two = default_ns2_kernel(precision == MLMC_FP32_PATH, pay, M, nf, scheme, false, kGdThreads);
+    const void *whole = two && !anti ? two : pick(mt, false, nf > kLongLaneSteps, false);
     if (!whole) return fail(MLMC_EINVAL, "no kernel for payoff %d", pay);
     rc = max_resident_blocks(whole, kGdThreads, &out->resident[kVarWhole]);
     if (rc) return rc;
@@ -428,6 +427,7 @@ int level_kernels(int l, int M, int precision, const mlmc_model *model, const ml
     if (anti) {
         const void *ak = precision == MLMC_FP32_PATH ? level_anti_kernel_fp32(pay, mt, scheme, nf > kLongLaneSteps)
                                                      : level_anti_kernel_fp64(pay, mt, scheme, nf > kLongLaneSteps);
+        if (const void *k = default_ns2_kernel(precision == MLMC_FP32_PATH, pay, M, nf, scheme, true, kGdThreads)) ak = k;
         if (!ak) return fail(MLMC_EINVAL, "no antithetic kernel for payoff %d", pay);
         int ra = 0;
         rc = max_resident_blocks(ak, kGdThreads, &ra);

@@ -20,6 +20,7 @@
 
 #include "engine.h"
 #include "normal64.cuh"
+#include "packed.cuh"
 #include "rng.cuh"
 
 namespace mlmcgb {
@@ -578,6 +579,124 @@ __device__ __forceinline__ void simulate_multi(const LevelParams &p, uint32_t s_
     }
 }
 
+// Two FP32 samples' paths in lockstep over the Philox calls [j0, j1) on packed pairs (sample 0 in the
+// low half): the operations and roundings of simulate_steps and simulate_multi, two samples per
+// instruction for the uniforms, the angles, the steps and the running sums (maxima and the MUFU
+// operations have no packed form).  States start at 1.  LO: running minima (split paths whose factors
+// may be negative).  The radius sqrt(-2 ln u) enters with its sign in the step's scale: d and the
+// coarse sum see the same products, and a negated product rounds like the product.
+template <int PAY, bool ANTI> struct PairState {
+    f32x2 S, sum;        // value, sum of values (Asian)
+    float hi[2], lo[2];  // maxima, minima (lookback)
+    __device__ __forceinline__ void init()
+    {
+        S = f2_splat(1.f);
+        sum = f2_splat(0.f);
+        hi[0] = hi[1] = lo[0] = lo[1] = 1.f;
+    }
+    template <bool LO> __device__ __forceinline__ void step(f32x2 d)
+    {
+        S = f2_fma(S, d, S);
+        if constexpr (PAY == kAsian) sum = f2_add(sum, S);
+        if constexpr (PAY == kLookback) {
+            float a, b;
+            f2_unpack(S, a, b);
+            hi[0] = fmaxf(hi[0], a);
+            hi[1] = fmaxf(hi[1], b);
+            if constexpr (LO) {
+                lo[0] = fminf(lo[0], a);
+                lo[1] = fminf(lo[1], b);
+            }
+        }
+    }
+};
+// Calls per iteration of the whole-path loops.
+template <int PAY, bool MIL, bool ANTI> constexpr int kPairUnroll = PAY == kLookback && !MIL && !ANTI ? 2 : 4;
+template <int MT, int PAY, bool MIL, bool RK, bool ANTI, bool LONG, bool LO, int UNROLL>
+__device__ __forceinline__ void simulate_pair(const LevelParams &p, const uint32_t s_hi[2], const uint32_t s_lo[2],
+                                              int j0, int j1, PairState<PAY, ANTI> &f, PairState<PAY, ANTI> &c,
+                                              PairState<PAY, ANTI> &a)
+{
+    const int M = MT ? MT : p.M;
+    const float a1 = (float)p.a;
+    const f32x2 rh = f2_splat(MIL ? (float)(p.rh - p.c2) : (float)p.rh), rH = f2_splat((float)(M * (p.rh - p.c2)));
+    const f32x2 minus_a = f2_splat(MIL ? -a1 : -(a1 * kSqrt2Ln2)), c2 = f2_splat((float)p.c2);
+    f.init();
+    c.init();
+    if constexpr (ANTI) a.init();
+    f32x2 dc = f2_splat(0.f);
+    int q = 0;
+    auto unit = [](uint32_t x) { return __uint_as_float((x & 0x007FFFFFu) | 0x3F800000u); };
+    // the increments d (Milstein: the normals with their sign reversed) of one word pair of both samples
+    auto normals = [&](uint32_t xa0, uint32_t xa1, uint32_t xb0, uint32_t xb1, f32x2 &d0, f32x2 &d1) {
+        float u0, u1, t0, t1;
+        f2_unpack(f2_fma(f2_pack(unit(xa0), unit(xa1)), f2_splat(-1.f), f2_splat(2.f)), u0, u1);
+        f2_unpack(f2_fma(f2_pack(unit(xb0), unit(xb1)), f2_splat(-6.28318530717958647692f),
+                         f2_splat(9.42477796076937971538f)), t0, t1);
+        auto sine = [&]() { return f2_pack(sin_approx(t0), sin_approx(t1)); };
+        auto cosine = [&]() { return f2_pack(cos_approx(t0), cos_approx(t1)); };
+        if constexpr (MIL) {
+            float l0, l1;
+            f2_unpack(f2_mul(f2_pack(lg2_approx(u0), lg2_approx(u1)), f2_splat(-1.38629436111989061883f)), l0, l1);
+            const f32x2 r = f2_pack(sqrt_approx(l0), sqrt_approx(l1));
+            const f32x2 sn = sine(), cs = cosine();
+            d0 = f2_mul(r, cs);
+            d1 = f2_mul(r, sn);
+        } else {
+            const f32x2 ra = f2_mul(f2_pack(sqrt_approx(-lg2_approx(u0)), sqrt_approx(-lg2_approx(u1))), minus_a);
+            const f32x2 sn = sine(), cs = cosine();
+            d0 = f2_fma(ra, cs, rh);
+            d1 = f2_fma(ra, sn, rh);
+        }
+    };
+    auto call = [&](int j) {
+        const uint4 x = philox_of<RK>(p, make_uint4(p.ctr3, (uint32_t)j, s_hi[0], s_lo[0]));
+        const uint4 y = philox_of<RK>(p, make_uint4(p.ctr3, (uint32_t)j, s_hi[1], s_lo[1]));
+        f32x2 z[4], d[4];
+        normals(x.x, y.x, x.y, y.y, z[0], z[1]);
+        normals(x.z, y.z, x.w, y.w, z[2], z[3]);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) d[k] = MIL ? f2_fma(f2_fma(c2, z[k], minus_a), z[k], rh) : z[k];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            dc = (MT == 4 && k == 0) ? z[k] : f2_add(dc, z[k]);
+            f.template step<LO>(d[k]);
+            if constexpr (ANTI) a.template step<LO>(d[MT == 4 ? 3 - k : (k ^ 1)]);
+            bool coarse_now;
+            if constexpr (MT != 0) {
+                coarse_now = (k + 1) % MT == 0;
+            } else {
+                coarse_now = ++q == M;
+                if (coarse_now) q = 0;
+            }
+            if (coarse_now) {
+                c.template step<LO>(MIL ? f2_fma(f2_fma(c2, dc, minus_a), dc, rH) : dc);
+                dc = f2_splat(0.f);
+            }
+        }
+    };
+    if constexpr (!(LONG && PAY == kAsian)) {
+#pragma unroll UNROLL
+        for (int j = j0; j < j1; ++j) call(j);
+    } else {
+        f32x2 ft = f2_splat(0.f), ct = ft, at = ft;  // totals of the finished groups
+        for (int g = j0; g < j1; g += kSumGroup) {
+            const int ge = min(g + kSumGroup, j1);
+            for (int j = g; j < ge; ++j) call(j);
+            ft = f2_add(ft, f.sum);
+            ct = f2_add(ct, c.sum);
+            f.sum = c.sum = f2_splat(0.f);
+            if constexpr (ANTI) {
+                at = f2_add(at, a.sum);
+                a.sum = f2_splat(0.f);
+            }
+        }
+        f.sum = ft;
+        c.sum = ct;
+        if constexpr (ANTI) a.sum = at;
+    }
+}
+
 __device__ __forceinline__ double warp_sum(double v)
 {
 #pragma unroll
@@ -830,8 +949,32 @@ __device__ __forceinline__ void multi_samples(const LevelParams &p, uint32_t s_h
     }
     R fS[NS], fsum[NS], fhi[NS], fls[NS], cS[NS], csum[NS], chi[NS], cls[NS];
     R aS[NS], asum[NS], ahi[NS], als[NS];
-    simulate_multi<R, MT, PAY, MIL, NS, RK, CALLS, ANTI, LONG>(p, s_hi, s_lo, fS, fsum, fhi, fls, cS, csum, chi, cls,
-                                                               aS, asum, ahi, als);
+    if constexpr (NS == 2 && sizeof(R) == 4 && PAY != kGeoAsian) {
+        const uint32_t hi2[2] = {s_hi, s_hi};
+        PairState<PAY, ANTI> f, c, a;
+        simulate_pair<MT, PAY, MIL, RK, ANTI, LONG, false, CALLS ? 1 : kPairUnroll<PAY, MIL, ANTI>>(p, hi2, s_lo, 0, CALLS ? CALLS : p.nf >> 2, f,
+                                                                         c, a);
+        f2_unpack(f.S, fS[0], fS[1]);
+        f2_unpack(f.sum, fsum[0], fsum[1]);
+        f2_unpack(c.S, cS[0], cS[1]);
+        f2_unpack(c.sum, csum[0], csum[1]);
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            fhi[i] = f.hi[i];
+            chi[i] = c.hi[i];
+            fls[i] = cls[i] = R(0);
+        }
+        if constexpr (ANTI) {
+            f2_unpack(a.S, aS[0], aS[1]);
+            f2_unpack(a.sum, asum[0], asum[1]);
+            ahi[0] = a.hi[0];
+            ahi[1] = a.hi[1];
+            als[0] = als[1] = R(0);
+        }
+    } else {
+        simulate_multi<R, MT, PAY, MIL, NS, RK, CALLS, ANTI, LONG>(p, s_hi, s_lo, fS, fsum, fhi, fls, cS, csum, chi, cls,
+                                                                   aS, asum, ahi, als);
+    }
 #pragma unroll
     for (int i = 0; i < NS; ++i) {
         R Pf = path_payoff<R, PAY>(p, false, fS[i], fsum[i], fhi[i], fls[i], S0, logS0, inv_nf);
@@ -1229,13 +1372,16 @@ __global__ void __launch_bounds__(1024) level_kernel(const LevelParams p)
     finish_sums(m, p);
 }
 
-// Two samples per thread and iteration, one thread per sample (no split, no antithetic path): the
-// two samples' Philox and step chains are independent, so each scheduler has twice the
-// instruction-level parallelism per warp, at more registers (64 against 54).  A kernel of its own
-// (not a runtime branch of level_kernel) so that the one-sample kernels keep their register count;
-// at most 512 threads per block, which lets it hold up to 128 registers.
-template <typename R, int MT, int PAY, bool LONG = false>
-__global__ void __launch_bounds__(512) level_ns2_kernel(const LevelParams p)
+// Two samples per thread and iteration, one thread per sample (no split): the two samples' Philox and
+// step chains are independent, and their FP32 arithmetic runs on packed pairs (simulate_pair).  A
+// kernel of its own (not a runtime branch of level_kernel); at most 512 threads per block.  The call
+// loop's unroll keeps each kernel at 64 registers (kPairUnroll; a register cap on the longer loops
+// cost 3 %), the one-sample kernels' residency, hence their grid and the order of their sums.
+// Scalar two-sample kernels before: Asian level 6, 1e6 samples, 3.23 -> 3.01 ms, lookback 3.18 ->
+// 3.06 ms; one-sample kernels before: Asian level 4, 1e6 samples, Milstein 249 -> 224 us, antithetic
+// 250 -> 220 us, both 274 -> 242 us.
+template <typename R, int MT, int PAY, bool MIL = false, bool ANTI = false, bool LONG = false>
+__global__ void __launch_bounds__(512, LONG ? 2 : 0) level_ns2_kernel(const LevelParams p)
 {
     double m[4] = {0.0, 0.0, 0.0, 0.0};
     float b1 = 0.f, b2 = 0.f, b3 = 0.f, b4 = 0.f;
@@ -1243,11 +1389,11 @@ __global__ void __launch_bounds__(512) level_ns2_kernel(const LevelParams p)
     const uint64_t t = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x, T = (uint64_t)gridDim.x * blockDim.x;
     if (p.nf == 4) {
         if (p.y_out)
-            multi_range<R, MT, PAY, false, 2, true, 1, false, LONG>(p, p.first, p.N, t, T, m, b1, b2, b3, b4, nb, p.y_out);
+            multi_range<R, MT, PAY, MIL, 2, true, 1, ANTI, LONG>(p, p.first, p.N, t, T, m, b1, b2, b3, b4, nb, p.y_out);
         else
-            multi_range<R, MT, PAY, false, 2, true, 1, false, LONG>(p, p.first, p.N, t, T, m, b1, b2, b3, b4, nb, nullptr);
+            multi_range<R, MT, PAY, MIL, 2, true, 1, ANTI, LONG>(p, p.first, p.N, t, T, m, b1, b2, b3, b4, nb, nullptr);
     } else {
-        multi_range<R, MT, PAY, false, 2, true, 0, false, LONG>(p, p.first, p.N, t, T, m, b1, b2, b3, b4, nb, p.y_out);
+        multi_range<R, MT, PAY, MIL, 2, true, 0, ANTI, LONG>(p, p.first, p.N, t, T, m, b1, b2, b3, b4, nb, p.y_out);
     }
     fold_batch<R>(m, b1, b2, b3, b4);
     finish_sums(m, p);
@@ -1421,27 +1567,24 @@ template <typename R> const void *select_anti_kernel(int payoff, int mt, int sch
     return nullptr;
 }
 
-// Two-samples-per-thread kernels (Euler--Maruyama, one thread per sample, mt = 4 or 0).
-template <typename R, int MT> const void *select_ns2_by_payoff(int payoff, bool long_lanes)
+// Two-samples-per-thread kernels (one thread per sample, mt = 4 or 0).
+template <typename R, int MT, bool MIL, bool ANTI> const void *select_ns2_by_payoff(int payoff, bool long_lanes)
 {
     switch (payoff) {
-    case kEuropean: return (const void *)level_ns2_kernel<R, MT, kEuropean>;
+    case kEuropean: return (const void *)level_ns2_kernel<R, MT, kEuropean, MIL, ANTI>;
     case kAsian:
         if constexpr (kBlockedSum<R, kAsian>) {
-            if (long_lanes) return (const void *)level_ns2_kernel<R, MT, kAsian, true>;
+            if (long_lanes) return (const void *)level_ns2_kernel<R, MT, kAsian, MIL, ANTI, true>;
         }
-        return (const void *)level_ns2_kernel<R, MT, kAsian>;
-    case kLookback: return (const void *)level_ns2_kernel<R, MT, kLookback>;
-    case kDigital: return (const void *)level_ns2_kernel<R, MT, kDigital>;
-    case kLinear: return (const void *)level_ns2_kernel<R, MT, kLinear>;
-    case kGeoAsian: return (const void *)level_ns2_kernel<R, MT, kGeoAsian>;
-    default: return nullptr;
+        return (const void *)level_ns2_kernel<R, MT, kAsian, MIL, ANTI>;
+    case kLookback: return (const void *)level_ns2_kernel<R, MT, kLookback, MIL, ANTI>;
+    case kDigital: return (const void *)level_ns2_kernel<R, MT, kDigital, MIL, ANTI>;
+    default: break;
     }
-}
-template <typename R> const void *select_ns2_kernel(int payoff, int mt, bool long_lanes)
-{
-    if (mt == 4) return select_ns2_by_payoff<R, 4>(payoff, long_lanes);
-    if (mt == 0) return select_ns2_by_payoff<R, 0>(payoff, long_lanes);
+    if constexpr (!MIL && !ANTI) {
+        if (payoff == kLinear) return (const void *)level_ns2_kernel<R, MT, kLinear>;
+        if (payoff == kGeoAsian) return (const void *)level_ns2_kernel<R, MT, kGeoAsian>;
+    }
     return nullptr;
 }
 

@@ -15,6 +15,8 @@
 #pragma once
 #include <cstdint>
 
+#include "packed.cuh"
+
 namespace mlmcgb {
 
 constexpr int kHidden = 64;
@@ -67,39 +69,6 @@ __device__ __forceinline__ float tanh_approx(float x)
     asm("tanh.approx.f32 %0, %1;" : "=f"(y) : "f"(x));
     return y;
 }
-
-// Two FP32 values in one 64-bit register pair, for the packed FP32 arithmetic of sm_100 and
-// later (fma / mul / add .rn.f32x2: each half rounds exactly as the scalar instruction would).
-typedef unsigned long long f32x2;
-__device__ __forceinline__ f32x2 f2_pack(float lo, float hi)
-{
-    f32x2 r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
-    return r;
-}
-__device__ __forceinline__ void f2_unpack(f32x2 v, float &lo, float &hi)
-{
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
-}
-__device__ __forceinline__ f32x2 f2_fma(f32x2 a, f32x2 b, f32x2 c)
-{
-    f32x2 d;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
-    return d;
-}
-__device__ __forceinline__ f32x2 f2_mul(f32x2 a, f32x2 b)
-{
-    f32x2 d;
-    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-    return d;
-}
-__device__ __forceinline__ f32x2 f2_add(f32x2 a, f32x2 b)
-{
-    f32x2 d;
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-    return d;
-}
-__device__ __forceinline__ f32x2 f2_splat(float v) { return f2_pack(v, v); }
 
 // 2 GELU(z) of both halves: u = z (sqrt(2/pi) + 0.044715 sqrt(2/pi) z^2), then z + z tanh(u)
 // (each half equals twice the scalar z/2 + (z/2) tanh(u) exactly).
