@@ -15,11 +15,12 @@
 //            function in IEEE floating-point arithmetic", ACM TOMS 16, 1990);
 //   sqrt     a 24-bit hardware reciprocal root, then one third-order correction
 //            p (1 + r/2 + 3 r^2/8), p = x y, r = 1 - p y (the binomial series of (1 - r)^(-1/2));
-//   cos, sin quadrant, 512 angles per quadrant by table, the remaining angle delta < pi/1024 by
-//            its Taylor series and the addition theorems.
+//   cos, sin quadrant, 512 angles per quadrant by table, the rotation by the remaining angle
+//            delta < pi/1024 as three shears with tan(delta / 2) and sin(delta) from their Taylor
+//            series (nine 32-bit products; the four of the addition theorems take twelve).
 //
 // Error (against quadruple precision, 3e6 random words and the edges of every reduction): cos and sin
-// 2^-59.6 rms and 2^-57 at most, rho 2^-58.7 rms, 2^-56.8 at most from rho = 1/2 on and 2^-53.7 at
+// 2^-59.1 rms and 2^-57 at most, rho 2^-58.7 rms, 2^-56.8 at most from rho = 1/2 on and 2^-53.7 at
 // most (next to u = 1, where rho itself is below 2^-4).  An FP64 normal of size 1 to 2 rounds by up to
 // 2^-53.
 #pragma once
@@ -169,21 +170,15 @@ MLMC_FX void fx_circle(uint32_t t, const uint64_t *tab, uint64_t &c, uint64_t &s
     const uint64_t U = fx_wide(Dh, Dh) + dl + dl;               // delta^2 / 2: 2^-79
     const uint32_t U1 = fx_shr_lo((uint32_t)U, (uint32_t)(U >> 32), 30);  // 2^-49
     const uint32_t U2 = fx_mulhi(U1, U1);                       // delta^4 / 4: 2^-66
-    // u = 1 - cos delta = U - U^2 / 6, v = sin delta = delta - delta (U / 3 - U^2 / 30): 2^-71
-    const uint64_t u = (uint64_t)((int64_t)(int32_t)fx_mulhi(U2, 0x2AAAAAABu) * -32 + (int64_t)(U >> 8));
-    const uint32_t g = fx_mulhi(U1, 0xAAAAAAABu) - fx_mulhi(U2, 2185u);  // 2^-50
-    const uint64_t v = D - (fx_wide(Dh, g) >> 18);
-    const uint32_t Ch = (uint32_t)(C >> 32), Cl = (uint32_t)C, Sh = (uint32_t)(S >> 32), Sl = (uint32_t)S;
-    const uint32_t uh = (uint32_t)(u >> 32), ul = (uint32_t)u, vh = (uint32_t)(v >> 32), vl = (uint32_t)v;
-    // cos = C - (C u + S v), sin = S + (C v - S u); products in units of 2^-69.  The sum of the cross
-    // products stays below 2^64: 2^30 2^32 twice, 2^32 2^30.7 and 2^32 2^21.4
-    const uint64_t xc = fx_wide(Ch, ul) + fx_wide(Sh, vl) + fx_wide(Sl, vh) + fx_wide(Cl, uh);
-    const uint64_t pc = fx_wide(Ch, uh) + fx_wide(Sh, vh) + (xc >> 32);
-    c = C - (pc >> 7);
-    const uint64_t xp = fx_wide(Ch, vl) + fx_wide(Cl, vh);
-    const uint64_t xm = fx_wide(Sh, ul) + fx_wide(Sl, uh);
-    const int64_t ps = (int64_t)((fx_wide(Ch, vh) + (xp >> 32)) - (fx_wide(Sh, uh) + (xm >> 32)));
-    s = S + (uint64_t)(ps >> 7);
+    // v = sin delta = delta - delta (U / 3 - U^2 / 30) in units of 2^-71 and w = tan(delta / 2) =
+    // delta / 2 + (delta / 2) (U / 6 + U^2 / 30) in units of 2^-72
+    const uint32_t U3 = fx_mulhi(U1, 0xAAAAAAABu), U30 = fx_mulhi(U2, 2185u);  // 2^-50
+    const uint64_t v = D - (fx_wide(Dh, U3 - U30) >> 18);
+    const uint64_t w = D + (fx_wide(Dh, (U3 >> 1) + U30) >> 18);
+    // the rotation by delta as three shears: c1 = C - w S, s = S + v c1, c = c1 - w s
+    const uint64_t c1 = C - (fx_mul64(w, S) >> 8);              // products in units of 2^-70, 2^-69
+    s = S + (fx_mul64(v, c1) >> 7);
+    c = c1 - (fx_mul64(w, s) >> 8);
 }
 // Signs of the cosine and sine of angle t as all-ones masks, and whether they trade places.
 MLMC_FX uint64_t fx_cos_sign(uint32_t t) { return (uint64_t)(int64_t)((int32_t)(t + 0x40000000u) >> 31); }
