@@ -147,11 +147,15 @@ struct BatchBuffers {
     }
 };
 
-// Fine steps per chunk of a round with `total` fine steps of new work: about four chunks per
-// resident block, at least 2^14 and at most 2^22 steps.
-double chunk_steps(double total, int blocks)
+// Fine steps per chunk of a round with `total` fine steps of new work: about eight chunks per SM, at
+// least 2^14 and at most 2^22 steps.  The number does not follow the kernel's residency, so that the
+// chunks, and with them the order of the FP32 sums, are the same for any build of it.
+int chunk_steps(double total, double *steps)
 {
-    return std::min(std::max(total / (4.0 * blocks), 16384.0), 4194304.0);
+    int sms = 0;
+    const int rc = device_sms(&sms);
+    if (!rc) *steps = std::min(std::max(total / (8.0 * sms), 16384.0), 4194304.0);
+    return rc;
 }
 
 // Append one task (samples [first, first + N) of `level` of one problem) and its chunks of about
@@ -258,7 +262,7 @@ extern "C" int mlmc_estimate_batch(int n, const mlmc_problem *problems, int M, i
         tasks.clear();
         chunks.clear();
         ranges.clear();
-        // total new work of the round sets the chunk size: about 4 chunks per resident block
+        // total new work of the round sets the chunk size: about 8 chunks per SM
         double total = 0.0;
         for (int i = 0; i < n; ++i) {
             if (!drv[i].active()) continue;
@@ -266,7 +270,12 @@ extern "C" int mlmc_estimate_batch(int n, const mlmc_problem *problems, int M, i
             for (int l = 0; l <= drv[i].finest_level(); ++l) total += (double)dN[l] * (double)ipow(M, l);
         }
         if (total == 0.0) break;
-        const double W = chunk_steps(total, blocks);
+        double W = 0.0;
+        rc = chunk_steps(total, &W);
+        if (rc) {
+            cleanup();
+            return rc;
+        }
         for (int i = 0; i < n; ++i) {
             if (!drv[i].active()) continue;
             const std::vector<uint64_t> &dN = drv[i].next_samples();
@@ -360,7 +369,9 @@ extern "C" int mlmc_level_sums_batch(int n, const mlmc_level_task *tasks, int M,
     std::vector<LevelParams> lp;
     std::vector<BatchChunk> chunks;
     std::vector<BatchRange> ranges;
-    const double W = chunk_steps(total, blocks);
+    double W = 0.0;
+    rc = chunk_steps(total, &W);
+    if (rc) return rc;
     uint64_t y_off = 0;
     std::vector<int> real;  // tasks with samples, in order
     for (int i = 0; i < n; ++i) {

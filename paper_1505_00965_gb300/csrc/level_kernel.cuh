@@ -256,7 +256,7 @@ __device__ __forceinline__ uint4 philox_of(const LevelParams &p, uint4 c)
 // exact sum of their fine d.  The caller checks p.fx, whose rule also keeps every factor positive;
 // no kGeoAsian (it needs every step's value).
 // Measured on the Asian call at level 5 (M = 4), 3.0e5 samples: 23.9 ms with the library's normals,
-// 3.12 ms with fixed-point normals and FP64 steps, 1.86 ms so (1.65e11 coupled steps/s).
+// 3.12 ms with fixed-point normals and FP64 steps, 1.75 ms so (1.75e11 coupled steps/s).
 template <typename R, int MT, int PAY, bool MIL, bool RK, bool ANTI, bool COARSE_LO>
 __device__ __forceinline__ void fx_steps(const LevelParams &p, uint32_t slo, uint32_t shi, int j0, int j1, R &fS_io,
                                          R &fsum_io, R &fhi_io, R &cS_io, R &csum_io, R &chi_io, R &clo_io,
@@ -1056,7 +1056,7 @@ __device__ __forceinline__ void multi_range(const LevelParams &p, uint64_t first
 // shuffles, t and T count whole warps and the loop exits are warp uniform.  Moments go into
 // m / b1..b4 / nb, and Y of sample first + i into y_out[i] when y_out is not NULL.
 template <typename R, int MT, int PAY, bool SPLIT, bool MIL, bool RK = true, bool ANTI = false,
-          bool LONG = false, bool POS = false>
+          bool LONG = false, bool POS = false, int NS = 1>
 __device__ __forceinline__ void regular_range(const LevelParams &p, uint64_t first, uint64_t N,
                                               uint64_t t, uint64_t T, double m[4], float &b1,
                                               float &b2, float &b3, float &b4, int &nb,
@@ -1072,7 +1072,7 @@ __device__ __forceinline__ void regular_range(const LevelParams &p, uint64_t fir
             else
                 multi_range<R, MT, PAY, MIL, 1, RK, 1, ANTI, LONG>(p, first, N, t, T, m, b1, b2, b3, b4, nb, nullptr);
         } else
-            multi_range<R, MT, PAY, MIL, 1, RK, 0, ANTI, LONG>(p, first, N, t, T, m, b1, b2, b3, b4, nb, y_out);
+            multi_range<R, MT, PAY, MIL, NS, RK, 0, ANTI, LONG>(p, first, N, t, T, m, b1, b2, b3, b4, nb, y_out);
     } else {
         static_assert(!ANTI, "antithetic paths run one thread per sample");
         const int P = p.lanes;
@@ -1415,6 +1415,10 @@ __global__ void __launch_bounds__(1024) level_small_kernel(const LevelParams p)
 
 // ------------------------------------------------------------------ batched rounds
 
+// Samples per thread of the batched kernel's whole paths: FP32 pairs (simulate_pair), the same samples
+// in the same order per thread.  The 96-problem batch: 357 -> 348 ms; three blocks per SM (80
+// registers) 352 ms.
+template <typename R> constexpr int kBatchSamples = sizeof(R) == 4 ? 2 : 1;
 // All samples of one chunk, by the threads of one block, on the code path of the chunk's task.
 // Y of sample first + i goes to y[i] when the task has per-sample output (p.y_out, indexed from
 // the task's first sample; NULL in the adaptive driver's rounds).
@@ -1437,7 +1441,7 @@ __device__ __forceinline__ void batch_chunk(const LevelParams &p, uint64_t first
     }
 #define MLMC_SMALL(PAY) small_range<R, PAY, false, false>(p, first, count, t, T, m, b1, b2, b3, b4, nb, y)
 #define MLMC_SPLIT(PAY) regular_range<R, MT, PAY, true, false, false>(p, first, count, t, T, m, b1, b2, b3, b4, nb, y)
-#define MLMC_PLAIN(PAY) regular_range<R, MT, PAY, false, false, false>(p, first, count, t, T, m, b1, b2, b3, b4, nb, y)
+#define MLMC_PLAIN(PAY) regular_range<R, MT, PAY, false, false, false, false, false, false, kBatchSamples<R>>(p, first, count, t, T, m, b1, b2, b3, b4, nb, y)
     if (p.small) {
         MLMC_BATCH_CASES(MLMC_SMALL)
     } else if (p.lanes > 1) {
@@ -1456,7 +1460,7 @@ __device__ __forceinline__ void batch_chunk(const LevelParams &p, uint64_t first
 // processed by one whole block with the same thread-to-sample mapping, so its sums do not
 // depend on which block claimed it.
 template <typename R, int MT>
-__global__ void __launch_bounds__(256) batch_kernel(const LevelParams *__restrict__ tasks,
+__global__ void __launch_bounds__(256, 2) batch_kernel(const LevelParams *__restrict__ tasks,
                                                     const BatchChunk *__restrict__ chunks,
                                                     const BatchHeader *__restrict__ header,
                                                     unsigned *counter, double *chunk_sums)
