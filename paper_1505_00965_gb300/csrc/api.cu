@@ -303,6 +303,22 @@ static int plan_idle(int level, int M, uint64_t N, int precision, const mlmc_mod
                                     : (double)std::max<uint64_t>(N, 1) * plan->lanes;
         while (plan->threads > 64 && plan->threads % 64 == 0 && std::ceil(items / plan->threads) < sms) plan->threads /= 2;
         if (plan->threads < 256) plan->blocks = std::max(1, (int)std::ceil(items / plan->threads));
+        // few, long FP32 paths: blocks whose other warps form the increments (one sample per lane group)
+        const double lane_warps = std::ceil(items / 32.0);
+        const int relay = relay_threads(lane_warps, nf / plan->lanes / 4, sms);
+        if (relay && precision == MLMC_FP32_PATH && payoff->estimator != MLMC_ANTITHETIC &&
+            !(launch && launch->samples_per_thread)) {
+            const bool split = plan->lanes > 1;
+            const void *k = level_relay_kernel_fp32(payoff->kind, M == 4 ? 4 : 0, split, model->scheme,
+                                                    nf / plan->lanes > kLongLaneSteps,
+                                                    split && positive_step_factors(model, level, M));
+            if (k) {
+                plan->kernel = k;
+                plan->threads = relay;
+                plan->blocks = (int)lane_warps;
+                plan->ns = 1;
+            }
+        }
     }
     return MLMC_OK;
 }

@@ -94,6 +94,21 @@ inline const void *default_ns2_kernel(int precision_is_fp32, int payoff, int M, 
     if (!precision_is_fp32 || M != 4 || nf < kNs2MinSteps || threads > kNs2MaxThreads) return nullptr;
     return level_ns2_kernel_fp32(payoff, 4, scheme, anti, nf > kLongLaneSteps);
 }
+// Launches of few, long FP32 paths (level_fp32_relay.cu): mt = 4 or 0, call and digital options; a block
+// of 128 or 256 threads per 32 lanes, NULL where there is none.
+const void *level_relay_kernel_fp32(int payoff, int mt, bool split, int scheme, bool long_lanes, bool positive);
+// Threads of their blocks for `lane_warps` warps of lanes of `calls` Philox calls on `sms` SMs; 0 where
+// the plain kernels are faster.  Timed against them on levels 4..8 at 4 to 1216 lane warps (152 SMs):
+// level 8 on 32 lanes 41 against 90 us up to 152 lane warps, 62 against 92 at 500, 86 against 105 at
+// 900, 104 against 106 at 1216; 64 calls per lane 19 against 25 us at 152, even at 900; whole paths of
+// 64 calls even at 400.  256 threads win up to about 400 lane warps (level 6 whole paths: 57 against 70
+// us at 152, 68 against 79 at 304, 111 against 108 at 500).
+inline int relay_threads(double lane_warps, long calls, int sms)
+{
+    const double per_sm = lane_warps / sms;
+    if (calls < 64 || per_sm > (calls < 128 ? 2.0 : 6.0)) return 0;
+    return per_sm <= 2.6 ? 256 : 128;
+}
 // The lanes-per-path model of both planners (plan_level and the device rounds): the time of w waves
 // of lane-items in whole waves (a partial last wave after whole ones costs min(1, kLanesTailSlope f
 // + kLanesTailBase) at fill f), a split step's cost relative to a whole-path one, and the least steps
