@@ -256,7 +256,7 @@ __device__ __forceinline__ uint4 philox_of(const LevelParams &p, uint4 c)
 // exact sum of their fine d.  The caller checks p.fx, whose rule also keeps every factor positive;
 // no kGeoAsian (it needs every step's value).
 // Measured on the Asian call at level 5 (M = 4), 3.0e5 samples: 23.9 ms with the library's normals,
-// 3.12 ms with fixed-point normals and FP64 steps, 1.75 ms so (1.75e11 coupled steps/s).
+// 3.12 ms with fixed-point normals and FP64 steps, 1.66 ms so (1.85e11 coupled steps/s).
 template <typename R, int MT, int PAY, bool MIL, bool RK, bool ANTI, bool COARSE_LO>
 __device__ __forceinline__ void fx_steps(const LevelParams &p, uint32_t slo, uint32_t shi, int j0, int j1, R &fS_io,
                                          R &fsum_io, R &fhi_io, R &cS_io, R &csum_io, R &chi_io, R &clo_io,

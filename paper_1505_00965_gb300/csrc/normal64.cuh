@@ -15,12 +15,15 @@
 //            function in IEEE floating-point arithmetic", ACM TOMS 16, 1990);
 //   sqrt     a 24-bit hardware reciprocal root, then one third-order correction
 //            p (1 + r/2 + 3 r^2/8), p = x y, r = 1 - p y (the binomial series of (1 - r)^(-1/2));
-//   cos, sin quadrant, 512 angles per quadrant by table, the rotation by the remaining angle
-//            delta < pi/1024 as three shears with tan(delta / 2) and sin(delta) from their Taylor
-//            series (nine 32-bit products; the four of the addition theorems take twelve).
+//   cos, sin quadrant, 4096 angles per quadrant by table, the rotation by the remaining angle
+//            delta < pi/8192 as three shears with tan(delta / 2) and sin(delta) from their Taylor
+//            series (nine 32-bit products; the four of the addition theorems take twelve).  With this
+//            many angles the series' one further term is small enough for FP32, whose pipe idles:
+//            512 angles took seven more products of the multiplier, which bounds the paths (digital
+//            level 2, 1e7 samples: 0.902 -> 0.850 ms; Asian level 5, 3.0e5 samples: 1.759 -> 1.663 ms).
 //
 // Error (against quadruple precision, 3e6 random words and the edges of every reduction): cos and sin
-// 2^-59.1 rms and 2^-57 at most, rho 2^-58.7 rms, 2^-56.8 at most from rho = 1/2 on and 2^-53.7 at
+// 2^-61.2 rms and 2^-58.2 at most, rho 2^-58.7 rms, 2^-56.8 at most from rho = 1/2 on and 2^-53.7 at
 // most (next to u = 1, where rho itself is below 2^-4).  An FP64 normal of size 1 to 2 rounds by up to
 // 2^-53.
 #pragma once
@@ -67,6 +70,7 @@ MLMC_FX float fx_rsqrt(float x)
     return y;
 }
 MLMC_FX uint32_t fx_bits(float x) { return __float_as_uint(x); }
+MLMC_FX uint32_t fx_round(float x) { return __float2uint_rn(x); }
 MLMC_FX float fx_float(uint32_t x) { return __uint2float_rn(x); }
 // The high word of (hi, lo) << k and the low word of (hi, lo) >> k, k < 32.
 MLMC_FX uint32_t fx_shl_hi(uint32_t lo, uint32_t hi, int k) { return __funnelshift_l(lo, hi, k); }
@@ -85,6 +89,7 @@ MLMC_FX uint32_t fx_bits(float x)
     std::memcpy(&u, &x, sizeof(u));
     return u;
 }
+MLMC_FX uint32_t fx_round(float x) { return (uint32_t)std::llrint(x); }
 MLMC_FX float fx_float(uint32_t x) { return (float)x; }
 MLMC_FX uint32_t fx_shl_hi(uint32_t lo, uint32_t hi, int k) { return k ? (hi << k) | (lo >> (32 - k)) : hi; }
 MLMC_FX uint32_t fx_shr_lo(uint32_t lo, uint32_t hi, int k) { return k ? (lo >> k) | (hi << (32 - k)) : lo; }
@@ -161,24 +166,20 @@ MLMC_FX uint64_t fx_radius(uint32_t w, const uint64_t *tab)
 // q = t >> 30, (cos, sin) = (c, s), (-s, c), (-c, -s), (s, -c) for q = 0..3.
 MLMC_FX void fx_circle(uint32_t t, const uint64_t *tab, uint64_t &c, uint64_t &s)
 {
-    const uint32_t i = (t >> 21) & 511u;
-    const uint64_t C = tab[kFxCos + i], S = tab[kFxCos + 512 - i];
-    const uint32_t dt = t << 11;                                // delta = 2 pi dt 2^-43 < pi / 1024
-    const uint64_t D = fx_mul64x32(kFxTwoPi60, dt);             // delta: 2^-71
-    const uint32_t Dh = (uint32_t)(D >> 32);
-    const uint32_t dl = fx_mulhi((uint32_t)D, Dh);
-    const uint64_t U = fx_wide(Dh, Dh) + dl + dl;               // delta^2 / 2: 2^-79
-    const uint32_t U1 = fx_shr_lo((uint32_t)U, (uint32_t)(U >> 32), 30);  // 2^-49
-    const uint32_t U2 = fx_mulhi(U1, U1);                       // delta^4 / 4: 2^-66
-    // v = sin delta = delta - delta (U / 3 - U^2 / 30) in units of 2^-71 and w = tan(delta / 2) =
-    // delta / 2 + (delta / 2) (U / 6 + U^2 / 30) in units of 2^-72
-    const uint32_t U3 = fx_mulhi(U1, 0xAAAAAAABu), U30 = fx_mulhi(U2, 2185u);  // 2^-50
-    const uint64_t v = D - (fx_wide(Dh, U3 - U30) >> 18);
-    const uint64_t w = D + (fx_wide(Dh, (U3 >> 1) + U30) >> 18);
+    const uint32_t i = (t >> 18) & 4095u;
+    const uint64_t C = tab[kFxCos + i], S = tab[kFxCos + 4096 - i];
+    const uint32_t dt = t << 14;                                // delta = 2 pi dt 2^-46 < pi / 8192
+    const uint64_t D = fx_mul64x32(kFxTwoPi60, dt);             // delta: 2^-74
+    // sin delta = delta - e and tan(delta / 2) = (delta + e / 2) / 2 with e = delta^3 / 6 (the next terms
+    // are below 2^-61), itself below 2^-36.6 and so in FP32, in units of 2^-68
+    const float df = (float)(int32_t)(uint32_t)(D >> 32);       // 2^-42
+    const uint32_t e = fx_round(df * df * (df * (0x1p-58f / 6)));
+    const uint64_t v = D - ((uint64_t)e << 6);
+    const uint64_t w = D + ((uint64_t)e << 5);                  // tan(delta / 2): 2^-75
     // the rotation by delta as three shears: c1 = C - w S, s = S + v c1, c = c1 - w s
-    const uint64_t c1 = C - (fx_mul64(w, S) >> 8);              // products in units of 2^-70, 2^-69
-    s = S + (fx_mul64(v, c1) >> 7);
-    c = c1 - (fx_mul64(w, s) >> 8);
+    const uint64_t c1 = C - (fx_mul64(w, S) >> 11);             // products in units of 2^-73, 2^-72
+    s = S + (fx_mul64(v, c1) >> 10);
+    c = c1 - (fx_mul64(w, s) >> 11);
 }
 // Signs of the cosine and sine of angle t as all-ones masks, and whether they trade places.
 MLMC_FX uint64_t fx_cos_sign(uint32_t t) { return (uint64_t)(int64_t)((int32_t)(t + 0x40000000u) >> 31); }
@@ -268,17 +269,20 @@ __device__ __forceinline__ double fx_to_double_signed(int64_t x, int unit)
     const int hi = __double2hiint(d);
     return __hiloint2double(hi ? hi - (unit << 20) : 0, __double2loint(d));
 }
-// The block's copy of the tables (8.5 KB of shared memory, one instance per kernel), filled by
-// fx_load_tables, which ends with a block barrier.
+// The block's copy of the tables (37 KB of shared memory, one instance per kernel), filled by
+// fx_load_tables (16 bytes a copy, all of a thread's in flight together), which ends with a block barrier.
 __device__ __forceinline__ uint64_t *fx_tables()
 {
-    __shared__ uint64_t tables[kFxWords];
+    __shared__ alignas(16) uint64_t tables[kFxWords];
     return tables;
 }
 __device__ __forceinline__ void fx_load_tables()
 {
     uint64_t *t = fx_tables();
-    for (int i = threadIdx.x; i < kFxWords; i += blockDim.x) t[i] = kFxTables[i];
+    for (int i = 2 * threadIdx.x; i < kFxWords; i += 2 * blockDim.x)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;"
+                     :: "r"((uint32_t)__cvta_generic_to_shared(t + i)), "l"(kFxTables + i) : "memory");
+    asm volatile("cp.async.wait_all;" ::: "memory");
     __syncthreads();
 }
 #endif
