@@ -138,7 +138,7 @@ typedef struct mlmc_launch {
                               an unpaired last sample alone; the automatic grid is the same.  The
                               samples and their Y are the same; the FP32 moment sums add them in
                               another order.  Automatic: 2 for FP32 Euler--Maruyama whole paths
-                              with M = 4 and M^l >= 16, else 1 (or the autotuner's choice). */
+                              with M = 4 and M^l >= 4, else 1 (or the autotuner's choice). */
 } mlmc_launch;
 
 /* Message describing the last failure on this host thread ("" if none). */

@@ -85,10 +85,12 @@ const void *level_anti_kernel_fp64(int payoff, int mt, int scheme, bool long_lan
 const void *level_ns2_kernel_fp32(int payoff, int mt, int scheme, bool anti, bool long_lanes);
 const void *level_ns2_kernel_fp32_other(int payoff, int mt, int scheme, bool anti, bool long_lanes);
 constexpr int kNs2MaxThreads = 512;
-// The planners' default of two samples per thread: FP32 whole paths with M = 4 and at least 16 fine
-// steps.  The two-sample kernel takes the same samples per thread in the same order on the same grid
-// (a thread's unpaired last sample runs alone).
-constexpr long kNs2MinSteps = 16;
+// The planners' default of two samples per thread: FP32 whole paths with M = 4 and at least one Philox
+// block.  The two-sample kernel takes the same samples per thread in the same order on the same grid
+// (a thread's unpaired last sample runs alone).  One block (level 1), 4e7 samples, one against two:
+// European 155.9 / 149.7 us, Asian 164.0 / 159.8, lookback 160.3 / 155.5, digital 179.8 / 172.3,
+// Milstein 171.5-194.8 / 162.3-182.3, antithetic 166.0-194.2 / 159.6-188.6; even at 2e6 and below.
+constexpr long kNs2MinSteps = 4;
 inline const void *default_ns2_kernel(int precision_is_fp32, int payoff, int M, long nf, int scheme, bool anti, int threads)
 {
     if (!precision_is_fp32 || M != 4 || nf < kNs2MinSteps || threads > kNs2MaxThreads) return nullptr;
