@@ -135,12 +135,12 @@ def _oracle_job(args):
 TRAFFIC_BYTES_PER_LAUNCH = 97280
 TRAFFIC_BASIS = ("ncu dram__bytes_read.sum + dram__bytes_write.sum of one level_ns2_kernel launch (lookback, "
                  "level 6, N=1e6, 608 blocks); algorithmic bytes 19.5 KB of block partials")
-# FP64 instructions (DFMA + DADD + DMUL, thread level) per coupled step of the FP64 Asian kernel, from
-# ncu's per-opcode counters on one launch (level 6, N = 1e5, one thread per sample).
-FP64_INSTR_PER_STEP = 36.51
-FP64_INSTR_BASIS = ("ncu smsp__sass_thread_inst_executed_op_{dfma,dadd,dmul}_pred_on of one level_kernel<double> "
-                    "launch (Asian, level 6, N=1e5): 20.76 + 8.26 + 7.50 per coupled step; deeper and shallower "
-                    "levels differ by their per-sample share")
+# Widening 32-bit integer products per coupled step of the FP64 paths (normals and step products are
+# 64-bit fixed point): a Philox block of four steps takes 20 in its rounds, 34 in each of its two pairs of
+# normals and 12 in the product of its four factors.
+FP64_PRODUCTS_PER_STEP = (20 + 2 * 34 + 12) / 4
+FP64_PRODUCTS_BASIS = ("counted from the source: 20 Philox, 2 x 34 normals, 12 step products per block of four "
+                       "fine steps; shifts and moves that run on the same pipe are not counted")
 
 ORACLE_SAMPLE = dict(eps=2e-2, seeds=tuple(range(1, 9)))
 ORACLE_SAMPLE_TEXT = ("oracle adaptive MLMC of the same two options and model at eps=2e-2 (not 1e-3), "
@@ -479,22 +479,23 @@ def gpu_arm(args) -> None:
         roofline["sfu"] = {"unavailable": str(exc)[:200]}
 
     # plain FP64 GPU MLMC on the same GPU, same eps (outside the timed region; Asian, the rank's
-    # eight seeds, median as for FP32), and its kernels against the FP64 pipe's measured rate
+    # eight seeds, median as for FP32), and its kernels against the integer multiplier's measured rate
     fp64_runs = [mlmc.mlmc_estimate(EPS, problems["asian"], s, M=M, Lmin=LMIN, Lmax=LMAX, N0=N0, precision="fp64",
                                     stream=stream) for s in seeds]
     fp64_ms = statistics.median(r.wall_ms for r in fp64_runs)
     fp32_asian_median = statistics.median(tte["asian"])
     fp64_steps = sum(r.path_steps for r in fp64_runs)
     fp64_kern_s = sum(r.kernel_ms for r in fp64_runs) / 1e3
-    roofline_fp64 = {"bound": "fp64", "kernel": "level_kernel<double> and level_small_kernel<double> (FP64 paths, "
+    roofline_fp64 = {"bound": "int_multiply", "kernel": "level_kernel<double> and level_small_kernel<double> (FP64 paths, "
                                                 "Asian, all levels of the eight estimates)",
-                     "path_steps_per_s": fp64_steps / fp64_kern_s, "unit": "FP64 instructions/s",
-                     "fp64_instructions_per_step": FP64_INSTR_PER_STEP, "fp64_instructions_basis": FP64_INSTR_BASIS}
+                     "path_steps_per_s": fp64_steps / fp64_kern_s, "unit": "widening products/s",
+                     "products_per_step": FP64_PRODUCTS_PER_STEP, "products_basis": FP64_PRODUCTS_BASIS}
     try:
-        achieved64 = FP64_INSTR_PER_STEP * fp64_steps / fp64_kern_s
-        roofline_fp64.update({"achieved": achieved64, "peak": probe["dfma_per_s"], "frac": achieved64 / probe["dfma_per_s"],
-                              "peak_basis": f"probe_peaks.cu: {probe['dfma_per_sm_per_clk']:.3f} FP64 FMA per SM "
-                                            "per clock (one FP64 instruction per operation)"})
+        achieved64 = FP64_PRODUCTS_PER_STEP * fp64_steps / fp64_kern_s
+        roofline_fp64.update({"achieved": achieved64, "peak": probe["imad_wide_per_s"],
+                              "frac": achieved64 / probe["imad_wide_per_s"],
+                              "peak_basis": f"probe_peaks.cu: {probe['imad_wide_per_sm_per_clk']:.2f} widening "
+                                            "multiplies per SM per clock"})
     except Exception as exc:
         roofline_fp64["unavailable"] = str(exc)[:200]
     extras = {} if args.no_extras else side_workloads(mlmc, stream)

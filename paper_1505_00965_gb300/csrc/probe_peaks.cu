@@ -3,7 +3,9 @@
 //   mufu    the four hardware approximations of Box--Muller (lg2, sqrt, sin, cos), 8 independent
 //           chains per thread
 //   ffma    FP32 fused multiply-adds, 8 independent chains per thread
-//   dfma    FP64 fused multiply-adds, 8 independent chains per thread (the pipe of the FP64 paths)
+//   dfma    FP64 fused multiply-adds, 8 independent chains per thread
+//   imad    widening 32-bit integer multiplies, 8 independent chains per thread (the pipe of the
+//           FP64 paths, whose normals and step products are fixed point)
 //   philox  Philox4x32-10 blocks (the generator of the level kernels, key schedule in registers)
 // Each kernel runs `iters` rounds per thread on a grid of `blocks_per_sm` x SMs x 256 threads and
 // writes one word per thread (the buffer has exactly that many words), so that nothing is
@@ -72,6 +74,25 @@ __global__ void __launch_bounds__(256) dfma_probe(float *out, int iters)
     out[tid] = (float)s;
 }
 
+__global__ void __launch_bounds__(256) imad_probe(float *out, int iters, uint32_t a)
+{
+    const uint32_t tid = blockIdx.x * blockDim.x + threadIdx.x;
+    uint32_t v[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) v[k] = tid + 77u * (uint32_t)k + 1u;
+    for (int i = 0; i < iters; ++i) {
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {  // the xor runs on another pipe
+            const uint64_t p = (uint64_t)v[k] * a;
+            v[k] = (uint32_t)(p >> 32) ^ (uint32_t)p;
+        }
+    }
+    uint32_t s = 0;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) s ^= v[k];
+    out[tid] = (float)s;
+}
+
 __global__ void __launch_bounds__(256) philox_probe(float *out, int iters, uint32_t k0, uint32_t k1)
 {
     const uint32_t tid = blockIdx.x * blockDim.x + threadIdx.x;
@@ -97,14 +118,15 @@ int main()
     cudaEventCreate(&e0);
     cudaEventCreate(&e1);
     const int iters = 4096;
-    double rate[4] = {0, 0, 0, 0};
-    for (int which = 0; which < 4; ++which) {
+    double rate[5] = {0, 0, 0, 0, 0};
+    for (int which = 0; which < 5; ++which) {
         float best = 1e30f;
         for (int rep = 0; rep < 4; ++rep) {
             cudaEventRecord(e0);
             if (which == 0) mufu_probe<<<blocks, threads>>>(out, iters);
             else if (which == 1) ffma_probe<<<blocks, threads>>>(out, iters);
             else if (which == 2) philox_probe<<<blocks, threads>>>(out, iters / 4, 1u, 2u);
+            else if (which == 4) imad_probe<<<blocks, threads>>>(out, iters, 0xCD9E8D57u);
             else dfma_probe<<<blocks, threads>>>(out, iters / 16);  // FP64 runs far slower than FP32
             cudaEventRecord(e1);
             cudaEventSynchronize(e1);
@@ -119,9 +141,10 @@ int main()
     const double per_sm_clk = 1.0 / ((double)sms * clock_khz * 1e3);
     printf("{\"sms\": %d, \"max_clock_mhz\": %.0f, \"mufu_per_s\": %.4e, \"mufu_per_sm_per_clk\": %.2f, "
            "\"ffma_per_s\": %.4e, \"ffma_per_sm_per_clk\": %.2f, \"philox_blocks_per_s\": %.4e, "
-           "\"dfma_per_s\": %.4e, \"dfma_per_sm_per_clk\": %.3f, \"status\": \"%s\"}\n",
+           "\"dfma_per_s\": %.4e, \"dfma_per_sm_per_clk\": %.3f, "
+           "\"imad_wide_per_s\": %.4e, \"imad_wide_per_sm_per_clk\": %.2f, \"status\": \"%s\"}\n",
            sms, clock_khz / 1e3, rate[0], rate[0] * per_sm_clk, rate[1], rate[1] * per_sm_clk, rate[2], rate[3],
-           rate[3] * per_sm_clk, cudaGetErrorString(err));
+           rate[3] * per_sm_clk, rate[4], rate[4] * per_sm_clk, cudaGetErrorString(err));
     cudaFree(out);
     return err == cudaSuccess ? 0 : 1;
 }
