@@ -285,10 +285,14 @@ bool positive_step_factors(const mlmc_model *m, int level, int M)
 }
 
 // Launches that leave most of the GPU idle (plan: the shape found so far, automatic fields zero in
-// launch).  Blocks shrink to 128 and 64 threads while the grid has fewer blocks than the GPU has SMs;
-// this regroups the FP64 partial sums only (every thread has one sample at most).  A warp that has its
+// launch).  FP32: blocks shrink to 128 and 64 threads while the grid has fewer blocks than the GPU has
+// SMs; this regroups the FP64 partial sums only (every thread has one sample at most).  A warp that has its
 // scheduler to itself runs a Philox call in about 245 cycles, two on one scheduler in about 305:
 // level 6 with 19,456 samples on whole paths 171 us with 256 threads, 121 with 64.
+// FP64: 128 threads where all blocks are resident and the fullest SM then has fewer threads.  A scheduler
+// is busy with a few of these warps, so the fullest SM sets the time; a block of 64 waits longer for its
+// 37 KB of tables, of which an SM holds six.  European level 4 with 1e4 samples 36.9 -> 34.8 us, level 1
+// 12.4 -> 10.4 (64 threads before); 1.9 waves (Asian level 5 with 3e5) take 1.66 ms on 256, 1.77 on 128.
 static int plan_idle(int level, int M, uint64_t N, int precision, const mlmc_model *model, const mlmc_payoff *payoff,
                      const mlmc_launch *launch, Plan *plan)
 {
@@ -301,8 +305,20 @@ static int plan_idle(int level, int M, uint64_t N, int precision, const mlmc_mod
     if (!tuned && !(launch && (launch->threads_per_block || launch->blocks))) {
         const double items = nf < 4 ? std::ceil((double)std::max<uint64_t>(N, 1) * nf / 4.0) + 1.0
                                     : (double)std::max<uint64_t>(N, 1) * plan->lanes;
-        while (plan->threads > 64 && plan->threads % 64 == 0 && std::ceil(items / plan->threads) < sms) plan->threads /= 2;
-        if (plan->threads < 256) plan->blocks = std::max(1, (int)std::ceil(items / plan->threads));
+        if (precision == MLMC_FP32_PATH) {
+            while (plan->threads > 64 && plan->threads % 64 == 0 && std::ceil(items / plan->threads) < sms) plan->threads /= 2;
+            if (plan->threads < 256) plan->blocks = std::max(1, (int)std::ceil(items / plan->threads));
+        } else {
+            constexpr int kThreads = 128;
+            int resident = 0;
+            if ((rc = max_resident_blocks(plan->kernel, kThreads, &resident))) return rc;
+            const double blocks = std::ceil(items / kThreads);
+            auto fullest = [&](int threads) { return std::ceil(std::ceil(items / threads) / sms) * threads; };
+            if (plan->threads > kThreads && blocks <= resident && fullest(kThreads) < fullest(plan->threads)) {
+                plan->threads = kThreads;
+                plan->blocks = std::max(1, (int)blocks);
+            }
+        }
         // few, long FP32 paths: blocks whose other warps form the increments (one sample per lane group)
         const double lane_warps = std::ceil(items / 32.0);
         const int relay = relay_threads(lane_warps, nf / plan->lanes / 4, sms);
