@@ -2,8 +2,8 @@
 //
 // The normals of one Philox block's word pair (xa, xb) are rho cos(2 pi u2), rho sin(2 pi u2) with
 // rho = sqrt(-2 ln u1) and 32-bit (or, on the FP32 path's stream, 23-bit) uniforms.  GB300 runs 2
-// FP64 operations per SM per clock against 32 widening 32-bit integer multiplies, 64 integer adds
-// and 16 MUFU operations (all measured), so one FP64 instruction costs as much as 16 widening
+// FP64 operations per SM per clock (1.65 measured) against 24 widening 32-bit integer multiplies, 64
+// integer adds and 16 MUFU operations, so one FP64 instruction costs as much as 12 or more widening
 // multiplies.  CUDA's double-precision log, sqrt and sincospi took 32 of the 36.5 FP64
 // instructions of a coupled step.  Here the whole pair is about 60 integer multiplies and no FP64:
 //
