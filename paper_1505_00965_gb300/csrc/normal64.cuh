@@ -5,7 +5,7 @@
 // FP64 operations per SM per clock (1.65 measured) against 24 widening 32-bit integer multiplies, 64
 // integer adds and 16 MUFU operations, so one FP64 instruction costs as much as 12 or more widening
 // multiplies.  CUDA's double-precision log, sqrt and sincospi took 32 of the 36.5 FP64
-// instructions of a coupled step.  Here the whole pair is about 60 integer multiplies and no FP64:
+// instructions of a coupled step.  Here the whole pair is 34 widening integer multiplies and no FP64:
 //
 //   ln u1    u = w 2^-32 with an integer w: w normalised to mu in [1/2, 1), c = k / 512 the
 //            multiple of 1/512 nearest 1 / mu (a hardware reciprocal), s = mu c - 1 exactly as a
