@@ -168,7 +168,7 @@ int plan_level(int level, int M, uint64_t N, int precision, int payoff, int sche
             rc = max_resident_blocks(kp, threads, &resp);
             if (rc) return rc;
             double best = 0.0;
-            const bool fp64 = precision != MLMC_FP32_PATH;
+            const bool fp64 = precision != MLMC_FP32_PATH && scheme != kLibrary;  // the model's two fits
             for (int P = 1; P <= 32; P *= 2) {
                 if (P > 1 && (nf % P != 0 || (nf / P) % unit != 0 || nf / P < min_lane_steps(fp64))) break;
                 const double T = (double)(P == 1 ? res1 : resp) * threads;
@@ -308,7 +308,7 @@ static int plan_idle(int level, int M, uint64_t N, int precision, const mlmc_mod
         if (precision == MLMC_FP32_PATH) {
             while (plan->threads > 64 && plan->threads % 64 == 0 && std::ceil(items / plan->threads) < sms) plan->threads /= 2;
             if (plan->threads < 256) plan->blocks = std::max(1, (int)std::ceil(items / plan->threads));
-        } else {
+        } else if (path_scheme(true, model->scheme, payoff->estimator == MLMC_SINGLE_LEVEL, nf) != kLibrary) {
             constexpr int kThreads = 128;
             int resident = 0;
             if ((rc = max_resident_blocks(plan->kernel, kThreads, &resident))) return rc;
@@ -342,16 +342,18 @@ static int plan_idle(int level, int M, uint64_t N, int precision, const mlmc_mod
 int plan_problem(int level, int M, uint64_t N, int precision, const mlmc_model *model, const mlmc_payoff *payoff,
                  const mlmc_launch *launch, Plan *plan, bool spread)
 {
+    const int scheme = path_scheme(precision != MLMC_FP32_PATH, model->scheme,
+                                   payoff->estimator == MLMC_SINGLE_LEVEL, ipow(M, level));
     if (model->kind == MLMC_MODEL_QUINTIC_ODE) return plan_ode(level, M, N, precision, model->scheme, launch, plan);
     if (payoff->estimator != MLMC_ANTITHETIC) {
-        const int rc = plan_level(level, M, N, precision, payoff->kind, model->scheme, launch, plan);
+        const int rc = plan_level(level, M, N, precision, payoff->kind, scheme, launch, plan);
         if (rc) return rc;
         // split lookback paths whose chunks all start above zero keep no running minimum
         if (plan->lanes > 1 && payoff->kind == kLookback && positive_step_factors(model, level, M)) {
             const int mt = M == 4 ? 4 : 0;
             const void *k = precision == MLMC_FP32_PATH
-                                ? level_kernel_fp32(payoff->kind, mt, true, model->scheme, false, true)
-                                : level_kernel_fp64(payoff->kind, mt, true, model->scheme, false, true);
+                                ? level_kernel_fp32(payoff->kind, mt, true, scheme, false, true)
+                                : level_kernel_fp64(payoff->kind, mt, true, scheme, false, true);
             if (k) plan->kernel = k;
         }
         return spread ? plan_idle(level, M, N, precision, model, payoff, launch, plan) : MLMC_OK;
@@ -366,15 +368,15 @@ int plan_problem(int level, int M, uint64_t N, int precision, const mlmc_model *
     mlmc_launch one = launch ? *launch : mlmc_launch{0, 0, 0, 0};
     one.lanes_per_path = 1;
     one.samples_per_thread = 1;
-    int rc = plan_level(level, M, N, precision, payoff->kind, model->scheme, &one, plan);
+    int rc = plan_level(level, M, N, precision, payoff->kind, scheme, &one, plan);
     if (rc) return rc;
     if (ipow(M, level) < 4) return spread ? plan_idle(level, M, N, precision, model, payoff, launch, plan) : MLMC_OK;
     const int mt = M == 4 ? 4 : 0;
     const bool long_lanes = ipow(M, level) > kLongLaneSteps;
-    plan->kernel = precision == MLMC_FP32_PATH ? level_anti_kernel_fp32(payoff->kind, mt, model->scheme, long_lanes)
-                                               : level_anti_kernel_fp64(payoff->kind, mt, model->scheme, long_lanes);
+    plan->kernel = precision == MLMC_FP32_PATH ? level_anti_kernel_fp32(payoff->kind, mt, scheme, long_lanes)
+                                               : level_anti_kernel_fp64(payoff->kind, mt, scheme, long_lanes);
     if (!(launch && launch->samples_per_thread)) {
-        const void *k = default_ns2_kernel(precision == MLMC_FP32_PATH, payoff->kind, M, ipow(M, level), model->scheme, true,
+        const void *k = default_ns2_kernel(precision == MLMC_FP32_PATH, payoff->kind, M, ipow(M, level), scheme, true,
                                            plan->threads);
         if (k) plan->kernel = k;
     }

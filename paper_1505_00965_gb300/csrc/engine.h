@@ -9,6 +9,10 @@ namespace mlmcgb {
 // Payoff codes, equal to the public mlmc_payoff_kind values.
 enum : int { kEuropean = 0, kAsian = 1, kLookback = 2, kDigital = 3, kLinear = 100, kGeoAsian = 101 };
 
+// Time-stepping schemes of the level kernels: the public mlmc_scheme values of the GBM model, and Milstein
+// FP64 paths on the library's normals (path_scheme).
+enum : int { kEuler = 0, kMilstein = 1, kLibrary = 16 };
+
 // Everything one level launch needs, passed by value as the kernel argument.
 struct LevelParams {
     double S0;        // initial value
@@ -76,6 +80,23 @@ const void *level_kernel_fp32(int payoff, int mt, bool split, int scheme, bool l
 // Milstein kernels (level_fp32_mil.cu, level_fp64_mil.cu), selected by the two above.
 const void *level_kernel_fp32_milstein(int payoff, int mt, bool split, bool long_lanes, bool positive);
 const void *level_kernel_fp64_milstein(int payoff, int mt, bool split, bool long_lanes, bool positive);
+// The same kernels with FP64 steps on the CUDA library's normals (level_fp64_library.cu).
+const void *level_kernel_fp64_library(int payoff, int mt, bool split, bool long_lanes, bool positive);
+const void *level_anti_kernel_fp64_library(int payoff, int mt, bool long_lanes);
+// FP64 Milstein paths of more than 1024 fine steps take the library's logarithm, root and sine, and FP64
+// steps, operation for operation.  P_l - P_{l-1} of strong order 1 shrinks like 1 / n while the rounding
+// of its two paths grows like sqrt(n): at 4096 steps a level's sums agree to 1e-9 only between forms that
+// round alike.  Against that form, over 57 cases each of 1e5 to 2.5e8 steps, S0 = K = 100, r = 0.05,
+// sigma = 0.2, the largest difference of the four sums with fixed-point normals and steps was 2.4e-11 on
+// M = 4 level 5, 7e-11 on M = 2 level 10, 6e-10 on level 11 (9 cases above 1e-10), 2.2e-9 and 4.4e-9 at 4096
+// steps and 2e-7 at 65536 (with fixed-point normals alone 8e-9 there); the strong order 1/2 of
+// Euler--Maruyama, coupled or antithetic, keeps all of its levels below 8e-10.  The single-level
+// estimator has no such difference.
+constexpr long kMilsteinFixedSteps = 1024;
+inline int path_scheme(bool fp64, int scheme, bool single_level, long nf)
+{
+    return fp64 && scheme == kMilstein && !single_level && nf > kMilsteinFixedSteps ? kLibrary : scheme;
+}
 // Antithetic level kernels (level_anti_fp32.cu, level_anti_fp64.cu): mt = 4 (M = 4) or 0 (M = 2).
 const void *level_anti_kernel_fp32(int payoff, int mt, int scheme, bool long_lanes);
 const void *level_anti_kernel_fp64(int payoff, int mt, int scheme, bool long_lanes);

@@ -5,6 +5,7 @@
 namespace mlmcgb {
 const void *level_anti_kernel_fp64(int payoff, int mt, int scheme, bool long_lanes)
 {
+    if (scheme == kLibrary) return level_anti_kernel_fp64_library(payoff, mt, long_lanes);
     return select_anti_kernel<double>(payoff, mt, scheme, long_lanes);
 }
 }  // namespace mlmcgb

@@ -7,6 +7,7 @@ namespace mlmcgb {
 // their own, compiled in parallel).
 const void *level_kernel_fp64(int payoff, int mt, bool split, int scheme, bool long_lanes, bool positive)
 {
+    if (scheme == kLibrary) return level_kernel_fp64_library(payoff, mt, split, long_lanes, positive);
     if (scheme == MLMC_MILSTEIN) return level_kernel_fp64_milstein(payoff, mt, split, long_lanes, positive);
     return select_scheme<double, false>(payoff, mt, split, long_lanes, positive);
 }

@@ -180,9 +180,9 @@ template <int PAY> __device__ __forceinline__ double rel_excess(const LevelParam
     if constexpr (PAY == kAsian) f = fma(fma(-0.5, S, sum), inv_n, 0.5 * inv_n);
     return positive_part(sub_rn(f, p.pay_k64));
 }
-template <typename R, int PAY> __device__ __forceinline__ R path_scale(const LevelParams &p, R Y)
+template <typename R, int PAY, int MIL> __device__ __forceinline__ R path_scale(const LevelParams &p, R Y)
 {
-    if constexpr (kRelExcess<R, PAY>) return mul_rn(R(p.pay_dS0_64), Y);
+    if constexpr (kRelExcess<R, PAY> && MIL != kLibrary) return mul_rn(R(p.pay_dS0_64), Y);
     else return Y;
 }
 
@@ -190,13 +190,13 @@ template <typename R, int PAY> __device__ __forceinline__ R path_scale(const Lev
 // inv_n; `coarse` picks the coarse path): a relative form above where it exists, else
 // payoff_value on the values times S0.  Differences and means of payoffs go through path_scale,
 // which applies the FP64 forms' common factor disc S0.
-template <typename R, int PAY>
+template <typename R, int PAY, int MIL>
 __device__ __forceinline__ R path_payoff(const LevelParams &p, bool coarse, R S, R sum, R hi, R ls, R S0, R logS0,
                                          R inv_n)
 {
     if constexpr (kRelPayoff<R, PAY>) {
         return rel_payoff<PAY>(p, coarse, S, sum, hi);
-    } else if constexpr (kRelExcess<R, PAY>) {
+    } else if constexpr (kRelExcess<R, PAY> && MIL != kLibrary) {
         return rel_excess<PAY>(p, S, sum, hi, inv_n);
     } else {
         const R n = coarse ? R(p.nf / p.M) : R(p.nf);
@@ -206,19 +206,27 @@ __device__ __forceinline__ R path_payoff(const LevelParams &p, bool coarse, R S,
 
 // Unit of the normals z that the step formulas below multiply: FP64 normals are the fixed-point
 // integers of fx_pair (units of 2^-58), converted to FP64 as they stand; the step scales sigma
-// sqrt(h) and sigma^2 h / 2 carry the unit (exact powers of two).
-template <typename R> __device__ __forceinline__ R step_a(const LevelParams &p)
+// sqrt(h) and sigma^2 h / 2 carry the unit (exact powers of two).  kLibrary: the library's normals.
+template <typename R, int MIL> __device__ __forceinline__ R step_a(const LevelParams &p)
 {
-    return sizeof(R) == 8 ? R(p.a * kFxZ) : R(p.a);
+    return sizeof(R) == 8 && MIL != kLibrary ? R(p.a * kFxZ) : R(p.a);
 }
-template <typename R> __device__ __forceinline__ R step_c2(const LevelParams &p)
+template <typename R, int MIL> __device__ __forceinline__ R step_c2(const LevelParams &p)
 {
-    return sizeof(R) == 8 ? R(p.c2 * kFxZ * kFxZ) : R(p.c2);
+    return sizeof(R) == 8 && MIL != kLibrary ? R(p.c2 * kFxZ * kFxZ) : R(p.c2);
 }
 // The four normals of a Philox block, in those units.
-template <typename R> __device__ __forceinline__ void block_normals(uint4 x, bool u23, R z[4])
+template <typename R, int MIL> __device__ __forceinline__ void block_normals(uint4 x, bool u23, R z[4])
 {
-    if constexpr (sizeof(R) == 8) {
+    if constexpr (MIL == kLibrary) {
+        R rho, c, s;
+        BoxMuller<R>::pair(x.x, x.y, rho, c, s, u23);
+        z[0] = rho * c;
+        z[1] = rho * s;
+        BoxMuller<R>::pair(x.z, x.w, rho, c, s, u23);
+        z[2] = rho * c;
+        z[3] = rho * s;
+    } else if constexpr (sizeof(R) == 8) {
         int64_t i[4];
         fx_pair(x.x, x.y, u23, fx_tables(), i[0], i[1]);
         fx_pair(x.z, x.w, u23, fx_tables(), i[2], i[3]);
@@ -257,7 +265,7 @@ __device__ __forceinline__ uint4 philox_of(const LevelParams &p, uint4 c)
 // no kGeoAsian (it needs every step's value).
 // Measured on the Asian call at level 5 (M = 4), 3.0e5 samples: 23.9 ms with the library's normals,
 // 3.12 ms with fixed-point normals and FP64 steps, 1.66 ms so (1.85e11 coupled steps/s).
-template <typename R, int MT, int PAY, bool MIL, bool RK, bool ANTI, bool COARSE_LO>
+template <typename R, int MT, int PAY, int MIL, bool RK, bool ANTI, bool COARSE_LO>
 __device__ __forceinline__ void fx_steps(const LevelParams &p, uint32_t slo, uint32_t shi, int j0, int j1, R &fS_io,
                                          R &fsum_io, R &fhi_io, R &cS_io, R &csum_io, R &chi_io, R &clo_io,
                                          R &aS_io, R &asum_io, R &ahi_io)
@@ -285,7 +293,7 @@ __device__ __forceinline__ void fx_steps(const LevelParams &p, uint32_t slo, uin
     int64_t dsum = 0;   // sum of the open coarse step's increments
     int64_t zsum = 0;   // Milstein: sum of its normals
     int q = 0;
-    const R a = step_a<R>(p), c2 = step_c2<R>(p), rHm = R(M * (p.rh - p.c2));
+    const R a = step_a<R, MIL>(p), c2 = step_c2<R, MIL>(p), rHm = R(M * (p.rh - p.c2));
     for (int j = j0; j < j1; ++j) {
         const uint4 x = philox_of<RK>(p, make_uint4(p.ctr3, (uint32_t)j, shi, slo));
         int64_t d[4], z[4];
@@ -344,20 +352,20 @@ __device__ __forceinline__ void fx_steps(const LevelParams &p, uint32_t slo, uin
 // coarse factor's d is the sum of the M fine ones.  Milstein (MIL): d = r h + sigma dW
 // + sigma^2 (dW^2 - h) / 2 = (r h - c2) + a z + c2 z^2 with a = sigma sqrt(h), c2 = sigma^2 h / 2,
 // and the coarse step the same formula on the summed increment with step M h.
-template <typename R, int MT, int PAY, bool SPLIT, bool MIL, bool RK = true, bool LONG = false, bool POS = false>
+template <typename R, int MT, int PAY, bool SPLIT, int MIL, bool RK = true, bool LONG = false, bool POS = false>
 __device__ __forceinline__ void simulate_steps(const LevelParams &p, uint32_t slo, uint32_t shi,
                                                int j0, int j1, PathAcc<R, PAY, SPLIT> &fa,
                                                PathAcc<R, PAY, SPLIT> &ca)
 {
-    if constexpr (sizeof(R) == 8 && PAY != kGeoAsian) {
+    if constexpr (sizeof(R) == 8 && PAY != kGeoAsian && MIL != kLibrary) {
         if (p.fx) {
             fx_steps<R, MT, PAY, MIL, RK, false, SPLIT && !POS>(p, slo, shi, j0, j1, fa.S, fa.sum, fa.hi, ca.S, ca.sum,
                                                                ca.hi, ca.lo, fa.lsum, fa.lsum, fa.lsum);
             return;
         }
     }
-    const R a = step_a<R>(p), rh = R(p.rh);
-    const R c2 = step_c2<R>(p), rhm = R(p.rh - p.c2);
+    const R a = step_a<R, MIL>(p), rh = R(p.rh);
+    const R c2 = step_c2<R, MIL>(p), rhm = R(p.rh - p.c2);
     R fS = fa.S, fsum = fa.sum, fhi = fa.hi, flo = fa.lo, fls = fa.lsum;
     R cS = ca.S, csum = ca.sum, chi = ca.hi, clo = ca.lo, cls = ca.lsum;
     R dc = R(0);
@@ -381,7 +389,7 @@ __device__ __forceinline__ void simulate_steps(const LevelParams &p, uint32_t sl
             d[2] = fma(ra, c, rh);
             d[3] = fma(ra, s, rh);
         } else {
-            block_normals<R>(x, u23, d);  // Milstein: d holds the normals until the steps below
+            block_normals<R, MIL>(x, u23, d);  // Milstein: d holds the normals until the steps below
             if constexpr (!MIL) {
 #pragma unroll
                 for (int k = 0; k < 4; ++k) d[k] = fma(a, d[k], rh);
@@ -441,7 +449,7 @@ __device__ __forceinline__ void simulate_steps(const LevelParams &p, uint32_t sl
 // at compile time (1 on levels with M^l = 4: straight-line code).  ANTI adds the antithetic fine
 // path (aS, asum, ahi, als): the same increments with each coarse step's M in reverse order
 // (M = 4: a Philox block is one coarse step, read backwards; M = 2: its two pairs swapped).
-template <typename R, int MT, int PAY, bool MIL, int NS, bool RK = true, int CALLS = 0, bool ANTI = false,
+template <typename R, int MT, int PAY, int MIL, int NS, bool RK = true, int CALLS = 0, bool ANTI = false,
           bool LONG = false>
 __device__ __forceinline__ void simulate_multi(const LevelParams &p, uint32_t s_hi, const uint32_t s_lo[NS], R fS[NS],
                                                R fsum[NS], R fhi[NS], R fls[NS], R cS[NS], R csum[NS],
@@ -449,8 +457,8 @@ __device__ __forceinline__ void simulate_multi(const LevelParams &p, uint32_t s_
                                                R als[NS])
 {
     static_assert(!ANTI || MT == 4 || MT == 0, "antithetic paths for M = 4 (MT = 4) and M = 2 (MT = 0)");
-    const R a = step_a<R>(p), rh = R(p.rh);
-    const R c2 = step_c2<R>(p), rhm = R(p.rh - p.c2);
+    const R a = step_a<R, MIL>(p), rh = R(p.rh);
+    const R c2 = step_c2<R, MIL>(p), rhm = R(p.rh - p.c2);
     const int M = MT ? MT : p.M;
     const R rHm = R(M * (p.rh - p.c2));
     const bool u23 = p.u23 != 0;
@@ -470,7 +478,7 @@ __device__ __forceinline__ void simulate_multi(const LevelParams &p, uint32_t s_
     }
     int q = 0;
     const int calls = CALLS ? CALLS : p.nf >> 2;
-    if constexpr (sizeof(R) == 8 && PAY != kGeoAsian) {
+    if constexpr (sizeof(R) == 8 && PAY != kGeoAsian && MIL != kLibrary) {
         static_assert(NS == 1, "FP64 paths run one at a time");
         if (p.fx) {
             fx_steps<R, MT, PAY, MIL, RK, ANTI, false>(p, s_lo[0], s_hi, 0, calls, fS[0], fsum[0], fhi[0], cS[0],
@@ -495,7 +503,7 @@ __device__ __forceinline__ void simulate_multi(const LevelParams &p, uint32_t s_
                 d[i][2] = fma(ra, c, rh);
                 d[i][3] = fma(ra, sn, rh);
             } else {
-                block_normals<R>(x, u23, d[i]);  // Milstein: d holds the normals until the steps below
+                block_normals<R, MIL>(x, u23, d[i]);  // Milstein: d holds the normals until the steps below
                 if constexpr (!MIL) {
 #pragma unroll
                     for (int k = 0; k < 4; ++k) d[i][k] = fma(a, d[i][k], rh);
@@ -611,8 +619,8 @@ template <int PAY, bool ANTI> struct PairState {
     }
 };
 // Calls per iteration of the whole-path loops.
-template <int PAY, bool MIL, bool ANTI> constexpr int kPairUnroll = PAY == kLookback && !MIL && !ANTI ? 2 : 4;
-template <int MT, int PAY, bool MIL, bool RK, bool ANTI, bool LONG, bool LO, int UNROLL>
+template <int PAY, int MIL, bool ANTI> constexpr int kPairUnroll = PAY == kLookback && !MIL && !ANTI ? 2 : 4;
+template <int MT, int PAY, int MIL, bool RK, bool ANTI, bool LONG, bool LO, int UNROLL>
 __device__ __forceinline__ void simulate_pair(const LevelParams &p, const uint32_t s_hi[2], const uint32_t s_lo[2],
                                               int j0, int j1, PairState<PAY, ANTI> &f, PairState<PAY, ANTI> &c,
                                               PairState<PAY, ANTI> &a)
@@ -838,7 +846,7 @@ __device__ __forceinline__ void join_chunks(const PathAcc<R, PAY, true> &A, int 
 
 // Y of sample s on a level with M^l >= 4, computed by the P lanes of one group (lane lig);
 // every lane of the group returns the same Y.
-template <typename R, int MT, int PAY, bool SPLIT, bool MIL, bool RK = true, bool LONG = false, bool POS = false>
+template <typename R, int MT, int PAY, bool SPLIT, int MIL, bool RK = true, bool LONG = false, bool POS = false>
 __device__ __forceinline__ R sample_Y(const LevelParams &p, uint64_t s, int lig, int P)
 {
     const uint32_t slo = (uint32_t)s, shi = (uint32_t)(s >> 32);
@@ -852,10 +860,10 @@ __device__ __forceinline__ R sample_Y(const LevelParams &p, uint64_t s, int lig,
     if constexpr (!SPLIT) {
         simulate_steps<R, MT, PAY, false, MIL, RK, LONG>(p, slo, shi, 0, p.nf >> 2, fa, ca);
         const R logS0 = PAY == kGeoAsian ? PathAcc<R, PAY, false>::log_r(S0) : R(0);
-        const R Pf = path_payoff<R, PAY>(p, false, fa.S, fa.sum, fa.hi, fa.lsum, S0, logS0, inv_nf);
-        if (p.fine_only) return path_scale<R, PAY>(p, Pf);
-        const R Pc = path_payoff<R, PAY>(p, true, ca.S, ca.sum, ca.hi, ca.lsum, S0, logS0, inv_nc);
-        return path_scale<R, PAY>(p, Pf - Pc);
+        const R Pf = path_payoff<R, PAY, MIL>(p, false, fa.S, fa.sum, fa.hi, fa.lsum, S0, logS0, inv_nf);
+        if (p.fine_only) return path_scale<R, PAY, MIL>(p, Pf);
+        const R Pc = path_payoff<R, PAY, MIL>(p, true, ca.S, ca.sum, ca.hi, ca.lsum, S0, logS0, inv_nc);
+        return path_scale<R, PAY, MIL>(p, Pf - Pc);
     } else {
         const int calls = (p.nf >> 2) / P;
         simulate_steps<R, MT, PAY, true, MIL, RK, LONG, POS>(p, slo, shi, lig * calls, (lig + 1) * calls, fa, ca);
@@ -878,7 +886,7 @@ __device__ __forceinline__ R sample_Y(const LevelParams &p, uint64_t s, int lig,
 // and the fifth moment operation took 2 (level 0) to 12 more.  The caller checks p.fx_fixed.  With the
 // shorter normals of the same change: adaptive Asian estimate at eps = 1e-3 (3.06e8 samples on level
 // 0, 8.6e7 on level 1) 9.37 -> 6.57 ms.
-template <typename R, int PAY, bool MIL> constexpr bool kFixedPayoff =
+template <typename R, int PAY, int MIL> constexpr bool kFixedPayoff =
     sizeof(R) == 8 && !MIL && (PAY == kEuropean || PAY == kAsian || PAY == kLookback);
 struct FixedMoments {
     __int128 s1 = 0;                     // sum of Y / (disc S0) in units of 2^-unit
@@ -933,7 +941,7 @@ template <int PAY> __device__ __forceinline__ int64_t fixed_block(const LevelPar
 
 // NS samples of one span run in lockstep: offsets i0, i0 + T, ... below n (the first always is),
 // sample indices (s_hi, lo0 + offset); moments go into m / b1..b4 / nb and Y into y_out[c0 + offset].
-template <typename R, int MT, int PAY, bool MIL, int NS, bool RK, int CALLS, bool ANTI, bool LONG>
+template <typename R, int MT, int PAY, int MIL, int NS, bool RK, int CALLS, bool ANTI, bool LONG>
 __device__ __forceinline__ void multi_samples(const LevelParams &p, uint32_t s_hi, uint32_t lo0, uint32_t i0,
                                               uint32_t T32, uint32_t n, uint64_t c0, R S0, R inv_nf, R inv_nc,
                                               R logS0, double m[4], float &b1, float &b2, float &b3,
@@ -977,13 +985,13 @@ __device__ __forceinline__ void multi_samples(const LevelParams &p, uint32_t s_h
     }
 #pragma unroll
     for (int i = 0; i < NS; ++i) {
-        R Pf = path_payoff<R, PAY>(p, false, fS[i], fsum[i], fhi[i], fls[i], S0, logS0, inv_nf);
+        R Pf = path_payoff<R, PAY, MIL>(p, false, fS[i], fsum[i], fhi[i], fls[i], S0, logS0, inv_nf);
         if constexpr (ANTI)
-            Pf = mul_rn(R(0.5), add_rn(Pf, path_payoff<R, PAY>(p, false, aS[i], asum[i], ahi[i], als[i], S0,
+            Pf = mul_rn(R(0.5), add_rn(Pf, path_payoff<R, PAY, MIL>(p, false, aS[i], asum[i], ahi[i], als[i], S0,
                                                                 logS0, inv_nf)));
         R Y = Pf;
-        if (!p.fine_only) Y -= path_payoff<R, PAY>(p, true, cS[i], csum[i], chi[i], cls[i], S0, logS0, inv_nc);
-        Y = path_scale<R, PAY>(p, Y);
+        if (!p.fine_only) Y -= path_payoff<R, PAY, MIL>(p, true, cS[i], csum[i], chi[i], cls[i], S0, logS0, inv_nc);
+        Y = path_scale<R, PAY, MIL>(p, Y);
         if (valid[i]) {
             if (y_out) y_out[c0 + i0 + (uint32_t)i * T32] = (double)Y;
             add_moments(Y, m, b1, b2, b3, b4, nb);
@@ -995,7 +1003,7 @@ __device__ __forceinline__ void multi_samples(const LevelParams &p, uint32_t s_h
 // below): thread t takes the offsets t, t + T, t + 2T, ... of each span, NS of them per iteration.
 // With NS = 2 a thread whose last offset has no partner runs it alone, so every thread takes the
 // same samples as with NS = 1 and the grid is the same; only the pairing differs.
-template <typename R, int MT, int PAY, bool MIL, int NS, bool RK = true, int CALLS = 0, bool ANTI = false,
+template <typename R, int MT, int PAY, int MIL, int NS, bool RK = true, int CALLS = 0, bool ANTI = false,
           bool LONG = false>
 __device__ __forceinline__ void multi_range(const LevelParams &p, uint64_t first, uint64_t N, uint64_t t,
                                             uint64_t T, double m[4], float &b1, float &b2, float &b3,
@@ -1055,7 +1063,7 @@ __device__ __forceinline__ void multi_range(const LevelParams &p, uint64_t first
 // groups of P = p.lanes lanes take one sample each, and since the lanes of a group join by
 // shuffles, t and T count whole warps and the loop exits are warp uniform.  Moments go into
 // m / b1..b4 / nb, and Y of sample first + i into y_out[i] when y_out is not NULL.
-template <typename R, int MT, int PAY, bool SPLIT, bool MIL, bool RK = true, bool ANTI = false,
+template <typename R, int MT, int PAY, bool SPLIT, int MIL, bool RK = true, bool ANTI = false,
           bool LONG = false, bool POS = false, int NS = 1>
 __device__ __forceinline__ void regular_range(const LevelParams &p, uint64_t first, uint64_t N,
                                               uint64_t t, uint64_t T, double m[4], float &b1,
@@ -1095,10 +1103,10 @@ __device__ __forceinline__ void regular_range(const LevelParams &p, uint64_t fir
 
 // The four normals z of Philox block q = (q_hi, q_lo) of a level with M^l < 4 and their step
 // increments d.
-template <typename R, bool MIL, bool RK = true>
+template <typename R, int MIL, bool RK = true>
 __device__ __forceinline__ void block_increments(const LevelParams &p, uint32_t q_hi, uint32_t q_lo, R z[4], R d[4])
 {
-    const R a = step_a<R>(p), rh = R(p.rh), c2 = step_c2<R>(p), rhm = R(p.rh - p.c2);
+    const R a = step_a<R, MIL>(p), rh = R(p.rh), c2 = step_c2<R, MIL>(p), rhm = R(p.rh - p.c2);
     const bool u23 = p.u23 != 0;
     const uint4 x = philox_of<RK>(p, make_uint4(p.ctr3, 0u, q_hi, q_lo));
     R rho, c, s;
@@ -1115,7 +1123,7 @@ __device__ __forceinline__ void block_increments(const LevelParams &p, uint32_t 
         d[3] = fma(ra, s, rh);
         return;
     }
-    block_normals<R>(x, u23, z);
+    block_normals<R, MIL>(x, u23, z);
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
         if constexpr (MIL) d[k] = fma(fma(c2, z[k], a), z[k], rhm);
@@ -1138,7 +1146,7 @@ template <typename R, int PAY> __device__ __forceinline__ Level0Consts<R> level0
     const double w = p.disc * p.S0 * (PAY == kAsian ? 0.5 : 1.0), base = p.disc * (p.S0 - p.K);
     const R floor = PAY == kLookback ? fmax(R(base), R(0)) : R(0);
     if constexpr (sizeof(R) == 4) return {R(w), R(base), floor};
-    else return {w * step_a<R>(p), fma(w, p.rh, base), floor};
+    else return {w * step_a<R, kEuler>(p), fma(w, p.rh, base), floor};
 }
 // Lookback: max(fma(max(d, 0), dS0, dS0mK), 0) = max(fma(d, dS0, dS0mK), max(dS0mK, 0)) exactly,
 // since dS0 > 0: for d > 0 the fma rounds to at least dS0mK, and for d <= 0 it rounds to at most
@@ -1152,14 +1160,14 @@ template <typename R> __device__ __forceinline__ R level0_payoff(R v, const Leve
 
 // The samples of Philox block q (slots r = 0 .. G - 1, sample q G + r) that lie in
 // [first, end), from the block's normals z and increments d.
-template <typename R, int PAY, bool MIL>
+template <typename R, int PAY, int MIL>
 __device__ __forceinline__ void small_block(const LevelParams &p, uint64_t q, uint64_t first, uint64_t end,
                                             const R z[4], const R d[4], double m[4], float &b1, float &b2,
                                             float &b3, float &b4, int &nb, double *y_out)
 {
     const int nf = p.nf;
     const uint32_t G = 4u / (uint32_t)nf;
-    const R a = step_a<R>(p), S0 = R(p.S0), c2 = step_c2<R>(p), rhm = R(p.rh - p.c2);
+    const R a = step_a<R, MIL>(p), S0 = R(p.S0), c2 = step_c2<R, MIL>(p), rhm = R(p.rh - p.c2);
     const R inv_nf = R(p.inv_nf), inv_nc = R(p.inv_nc);
     const R logS0 = PAY == kGeoAsian ? log(S0) : R(0);
     if (nf == 1 && q * 4 >= first && end - q * 4 >= 4) {
@@ -1231,7 +1239,7 @@ __device__ __forceinline__ void small_block(const LevelParams &p, uint64_t q, ui
 // Samples [first, first + N) of a level with M^l < 4.  G = 4 / M^l consecutive samples share
 // one Philox block: thread t takes blocks q = first / G + t, + T, ... and the G samples
 // q G .. q G + G - 1 that fall in the range; sample slot r takes normals r M^l .. of the block.
-template <typename R, int PAY, bool MIL, bool RK = true>
+template <typename R, int PAY, int MIL, bool RK = true>
 __device__ __forceinline__ void small_range(const LevelParams &p, uint64_t first, uint64_t N,
                                             uint64_t t, uint64_t T, double m[4], float &b1,
                                             float &b2, float &b3, float &b4, int &nb,
@@ -1359,10 +1367,10 @@ __device__ __forceinline__ void fold_batch(double m[4], float b1, float b2, floa
 // than kLongLaneSteps steps (two-level Asian sums); POS: split paths whose step factors 1 + d are
 // all positive (the host checks the bound of the normals), so that no chunk starts below zero
 // and the lookback lanes keep no running minimum.
-template <typename R, int MT, int PAY, bool SPLIT, bool MIL, bool ANTI = false, bool LONG = false, bool POS = false>
+template <typename R, int MT, int PAY, bool SPLIT, int MIL, bool ANTI = false, bool LONG = false, bool POS = false>
 __global__ void __launch_bounds__(1024) level_kernel(const LevelParams p)
 {
-    if constexpr (sizeof(R) == 8) fx_load_tables();
+    if constexpr (sizeof(R) == 8 && MIL != kLibrary) fx_load_tables();
     double m[4] = {0.0, 0.0, 0.0, 0.0};
     float b1 = 0.f, b2 = 0.f, b3 = 0.f, b4 = 0.f;  // FP32-path batch sums
     int nb = 0;
@@ -1382,7 +1390,7 @@ __global__ void __launch_bounds__(1024) level_kernel(const LevelParams p)
 // bit for bit.  One sample per lane group (the launch has at least as many groups as samples).  Asian
 // level 8, 1003 samples on 16 lanes: 159 us on the plain kernel with one warp per scheduler, 100 so.
 constexpr int kRelayCalls = 2, kRelayMaxWarps = 8;
-template <int MT, int PAY, bool SPLIT, bool MIL, bool LONG, bool POS>
+template <int MT, int PAY, bool SPLIT, int MIL, bool LONG, bool POS>
 __global__ void __launch_bounds__(32 * kRelayMaxWarps) level_relay_kernel(const LevelParams p)
 {
     using R = float;
@@ -1417,7 +1425,7 @@ __global__ void __launch_bounds__(32 * kRelayMaxWarps) level_relay_kernel(const 
                     const uint4 x = philox_of<true>(p, make_uint4(p.ctr3, (uint32_t)(j0 + min(jj, calls - 1)), shi, slo));
                     R d[4];
                     if constexpr (MIL) {
-                        block_normals<R>(x, false, d);
+                        block_normals<R, MIL>(x, false, d);
                     } else {
                         R rho, cs, sn;
                         box_muller_lg2(x.x, x.y, rho, cs, sn);
@@ -1481,8 +1489,8 @@ __global__ void __launch_bounds__(32 * kRelayMaxWarps) level_relay_kernel(const 
             Y = payoff_value<R, PAY>(tf, pf, hf, lf, inv_nf, p);
             if (!p.fine_only) Y = Y - payoff_value<R, PAY>(tc, pc, hc, lc, inv_nc, p);
         } else {
-            Y = path_payoff<R, PAY>(p, false, fS, fsum, fhi, fls, S0, R(0), inv_nf);
-            if (!p.fine_only) Y -= path_payoff<R, PAY>(p, true, cS, csum, chi, cls, S0, R(0), inv_nc);
+            Y = path_payoff<R, PAY, MIL>(p, false, fS, fsum, fhi, fls, S0, R(0), inv_nf);
+            if (!p.fine_only) Y -= path_payoff<R, PAY, MIL>(p, true, cS, csum, chi, cls, S0, R(0), inv_nc);
         }
         if (valid && lig == 0) {
             if (p.y_out) p.y_out[idx] = (double)Y;
@@ -1501,7 +1509,7 @@ __global__ void __launch_bounds__(32 * kRelayMaxWarps) level_relay_kernel(const 
 // Scalar two-sample kernels before: Asian level 6, 1e6 samples, 3.23 -> 3.01 ms, lookback 3.18 ->
 // 3.06 ms; one-sample kernels before: Asian level 4, 1e6 samples, Milstein 249 -> 224 us, antithetic
 // 250 -> 220 us, both 274 -> 242 us.
-template <typename R, int MT, int PAY, bool MIL = false, bool ANTI = false, bool LONG = false>
+template <typename R, int MT, int PAY, int MIL = false, bool ANTI = false, bool LONG = false>
 __global__ void __launch_bounds__(512, LONG ? 2 : 0) level_ns2_kernel(const LevelParams p)
 {
     double m[4] = {0.0, 0.0, 0.0, 0.0};
@@ -1521,7 +1529,7 @@ __global__ void __launch_bounds__(512, LONG ? 2 : 0) level_ns2_kernel(const Leve
 }
 
 // Levels with M^l < 4 (level 0, and level 1 when M = 2).
-template <typename R, int PAY, bool MIL>
+template <typename R, int PAY, int MIL>
 __global__ void __launch_bounds__(1024) level_small_kernel(const LevelParams p)
 {
     if constexpr (sizeof(R) == 8) fx_load_tables();
@@ -1615,7 +1623,7 @@ namespace mlmcgb {
 
 // The arithmetic-Asian kernel for lanes of `long_lanes` (more than kLongLaneSteps steps) or not;
 // the two are the same kernel where the sums keep one level (FP64 paths).
-template <typename R, int MT, bool SPLIT, bool MIL, bool ANTI> const void *asian_kernel(bool long_lanes)
+template <typename R, int MT, bool SPLIT, int MIL, bool ANTI> const void *asian_kernel(bool long_lanes)
 {
     if constexpr (kBlockedSum<R, kAsian>) {
         if (long_lanes) return (const void *)level_kernel<R, MT, kAsian, SPLIT, MIL, ANTI, true>;
@@ -1625,7 +1633,7 @@ template <typename R, int MT, bool SPLIT, bool MIL, bool ANTI> const void *asian
 
 // Kernel for (payoff, M specialisation, split, scheme, lane length) at precision R; nullptr for
 // an unknown payoff.
-template <typename R, int MT, bool SPLIT, bool MIL>
+template <typename R, int MT, bool SPLIT, int MIL>
 const void *select_by_payoff(int payoff, bool long_lanes, bool positive = false)
 {
     if constexpr (SPLIT) {
@@ -1642,7 +1650,7 @@ const void *select_by_payoff(int payoff, bool long_lanes, bool positive = false)
     }
 }
 
-template <typename R, bool MIL> const void *select_small_kernel(int payoff)
+template <typename R, int MIL> const void *select_small_kernel(int payoff)
 {
     switch (payoff) {
     case kEuropean: return (const void *)level_small_kernel<R, kEuropean, MIL>;
@@ -1656,7 +1664,7 @@ template <typename R, bool MIL> const void *select_small_kernel(int payoff)
 }
 
 // mt = -1 selects the kernel of levels with M^l < 4; MIL the Milstein kernels.
-template <typename R, bool MIL>
+template <typename R, int MIL>
 const void *select_scheme(int payoff, int mt, bool split, bool long_lanes, bool positive = false)
 {
     if (mt < 0) return select_small_kernel<R, MIL>(payoff);
@@ -1669,7 +1677,7 @@ const void *select_scheme(int payoff, int mt, bool split, bool long_lanes, bool 
 
 
 // Antithetic kernels: mt = 4 (M = 4) or 0 (M = 2), one thread per sample; nullptr otherwise.
-template <typename R, int MT, bool MIL> const void *select_anti_by_payoff(int payoff, bool long_lanes)
+template <typename R, int MT, int MIL> const void *select_anti_by_payoff(int payoff, bool long_lanes)
 {
     switch (payoff) {
     case kEuropean: return (const void *)level_kernel<R, MT, kEuropean, false, MIL, true>;
@@ -1693,7 +1701,7 @@ template <typename R> const void *select_anti_kernel(int payoff, int mt, int sch
 }
 
 // Two-samples-per-thread kernels (one thread per sample, mt = 4 or 0).
-template <typename R, int MT, bool MIL, bool ANTI> const void *select_ns2_by_payoff(int payoff, bool long_lanes)
+template <typename R, int MT, int MIL, bool ANTI> const void *select_ns2_by_payoff(int payoff, bool long_lanes)
 {
     switch (payoff) {
     case kEuropean: return (const void *)level_ns2_kernel<R, MT, kEuropean, MIL, ANTI>;
@@ -1714,7 +1722,7 @@ template <typename R, int MT, bool MIL, bool ANTI> const void *select_ns2_by_pay
 }
 
 // Relay kernels of the call and digital options; nullptr for the others.
-template <int MT, bool MIL> const void *select_relay(int payoff, bool split, bool long_lanes, bool positive)
+template <int MT, int MIL> const void *select_relay(int payoff, bool split, bool long_lanes, bool positive)
 {
     if (split) {
         switch (payoff) {

@@ -53,7 +53,7 @@ __global__ void __launch_bounds__(256) quintic_level_kernel(const LevelParams p)
         const uint64_t q = q0 + u;
         const uint4 w = philox4x32_10(make_uint4(p.ctr3, 0u, (uint32_t)(q >> 32), (uint32_t)q), p.rkey);
         R x0[4], xf[4], xc[4];
-        block_normals<R>(w, u23, x0);
+        block_normals<R, kEuler>(w, u23, x0);
 #pragma unroll
         for (int r = 0; r < 4; ++r) xf[r] = xc[r] = sizeof(R) == 8 ? x0[r] * R(kFxZ) : x0[r];
         quintic_paths<R, TAMED, 4>(xf, h, nf);

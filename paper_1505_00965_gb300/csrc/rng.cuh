@@ -112,4 +112,17 @@ __device__ __forceinline__ void box_muller_lg2(uint32_t xa, uint32_t xb, float &
 }
 constexpr float kSqrt2Ln2 = 1.17741002251547469101f;  // sqrt(2 ln 2)
 
+// FP64 normals of the kLibrary paths (engine.h): u = (x + 1) 2^-32 in (0, 1], CUDA's double-precision
+// log, sqrt and sincospi.  With u23 set, the FP32 stream's uniforms u = 1 - (x mod 2^23) 2^-23 instead.
+template <> struct BoxMuller<double> {
+    __device__ __forceinline__ static void pair(uint32_t xa, uint32_t xb, double &rho,
+                                                double &c, double &s, bool u23 = false)
+    {
+        const double u1 = u23 ? 1.0 - (double)(xa & 0x007FFFFFu) * 0x1p-23 : ((double)xa + 1.0) * 0x1p-32;
+        const double u2 = u23 ? 1.0 - (double)(xb & 0x007FFFFFu) * 0x1p-23 : ((double)xb + 1.0) * 0x1p-32;
+        rho = sqrt(-2.0 * log(u1));
+        sincospi(2.0 * u2, &s, &c);
+    }
+};
+
 }  // namespace mlmcgb
