@@ -567,7 +567,6 @@ int acquire_scratch(size_t ws_bytes, DriverScratch **out)
     s->device = dev;
     s->ws_bytes = ws_bytes;
     cudaError_t e = cudaMalloc(&s->ws, ws_bytes);
-    if (e == cudaSuccess) e = cudaMemset(s->ws, 0, ws_bytes);
     if (e == cudaSuccess) e = cudaMalloc(&s->d_sums, kDriverSumsPerLevel * MLMC_MAX_LEVELS * sizeof(double));
     if (e == cudaSuccess) e = cudaMallocHost(&s->h_sums, kDriverSumsPerLevel * MLMC_MAX_LEVELS * sizeof(double));
     if (e == cudaSuccess) e = cudaEventCreate(&s->ev0);
@@ -577,6 +576,10 @@ int acquire_scratch(size_t ws_bytes, DriverScratch **out)
         e = cudaStreamCreateWithFlags(&s->aux[k], cudaStreamNonBlocking);
         if (e == cudaSuccess) e = cudaEventCreateWithFlags(&s->join[k], cudaEventDisableTiming);
     }
+    // cleared and waited for on a stream of the set's own: nothing orders the caller's stream, which need
+    // not synchronise with the default stream, behind work queued there
+    if (e == cudaSuccess) e = cudaMemsetAsync(s->ws, 0, ws_bytes, s->aux[0]);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s->aux[0]);
     if (e != cudaSuccess) {
         free_scratch(s);
         return fail(MLMC_ECUDA, "driver setup failed: %s", cudaGetErrorString(e));

@@ -76,7 +76,8 @@ struct BatchBuffers {
         *this = BatchBuffers();
     }
 
-    int reserve(size_t tasks, size_t chunks)
+    // st: the stream of the rounds, on which a new counter is cleared
+    int reserve(size_t tasks, size_t chunks, cudaStream_t st)
     {
         if (tasks <= cap_tasks && chunks <= cap_chunks) return MLMC_OK;
         release();
@@ -92,7 +93,7 @@ struct BatchBuffers {
         CUDA_TRY(cudaMalloc(&d_chunk_sums, cap_chunks * 4 * sizeof(double)));
         CUDA_TRY(cudaMalloc(&d_task_sums, cap_tasks * 4 * sizeof(double)));
         CUDA_TRY(cudaMalloc(&d_counter, sizeof(unsigned)));
-        CUDA_TRY(cudaMemset(d_counter, 0, sizeof(unsigned)));
+        CUDA_TRY(cudaMemsetAsync(d_counter, 0, sizeof(unsigned), st));
         return MLMC_OK;
     }
 
@@ -286,7 +287,7 @@ extern "C" int mlmc_estimate_batch(int n, const mlmc_problem *problems, int M, i
                 refs.push_back({i, l});
             }
         }
-        rc = buf.reserve(tasks.size(), chunks.size());
+        rc = buf.reserve(tasks.size(), chunks.size(), st);
         if (rc) {
             cleanup();
             return rc;
@@ -386,7 +387,7 @@ extern "C" int mlmc_level_sums_batch(int n, const mlmc_level_task *tasks, int M,
     if (real.empty()) return MLMC_OK;
     cudaStream_t st = (cudaStream_t)stream;
     BatchBuffers buf;
-    rc = buf.reserve(lp.size(), chunks.size());
+    rc = buf.reserve(lp.size(), chunks.size(), st);
     if (!rc) {
         buf.header()->n_tasks = (uint32_t)lp.size();
         buf.header()->n_chunks = (uint32_t)chunks.size();

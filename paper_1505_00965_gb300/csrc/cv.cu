@@ -336,6 +336,7 @@ int mlmc_cv_set_params(mlmc_cv *cv, int level, const float *params, double kappa
         return fail(MLMC_EINVAL, "kappa must lie in [%g, %g]", kMinKappa, kMaxKappa);
     if (!cv->d_params[level]) CUDA_TRY(cudaMalloc(&cv->d_params[level], sizeof(float) * kNumParams));
     CUDA_TRY(cudaMemcpy(cv->d_params[level], params, sizeof(float) * kNumParams, cudaMemcpyHostToDevice));
+    CUDA_TRY(cudaStreamSynchronize(nullptr));  // a copy from pageable memory may return before it has arrived
     std::memcpy(cv->h_params[level], params, sizeof(float) * kNumParams);
     cv->info[level] = mlmc_cv_level_info();
     cv->info[level].trained = 1;
@@ -552,7 +553,7 @@ int mlmc_cv_train(int M, const mlmc_model *model, const mlmc_payoff *payoff, uin
         sd[l] = std::sqrt(std::max(v / (double)n_fit, 1e-300));
         float w[kNumParams];
         init_params(w, o.init_seed + 7919ull * (uint64_t)l);
-        CV_TRY(cudaMemcpy(d_P + kNumParams * l, w, sizeof(w), cudaMemcpyHostToDevice));
+        CV_TRY(cudaMemcpyAsync(d_P + kNumParams * l, w, sizeof(w), cudaMemcpyHostToDevice, st));
         targs.job[l] = TrainJob{X, Yd, d_P + kNumParams * l, (float)m, (float)(1.0 / sd[l])};
     }
     const auto t_data = std::chrono::steady_clock::now();

@@ -468,9 +468,10 @@ int level_kernels(int l, int M, int precision, const mlmc_model *model, const ml
         }                                                                                                   \
     } while (0)
 
-// Build the graph of one problem shape into `c` (kernels, residencies, nodes, slots, state).
+// Build the graph of one problem shape into `c` (kernels, residencies, nodes, slots, state; the slots
+// cleared on st, the stream of the first run).
 int gd_build(GdCache &c, int dev, const int key[10], int M, int Lmax, int precision, const mlmc_model *model,
-             const mlmc_payoff *payoff)
+             const mlmc_payoff *payoff, cudaStream_t st)
 {
     c.device = dev;
     std::memcpy(c.key, key, sizeof(c.key));
@@ -482,7 +483,7 @@ int gd_build(GdCache &c, int dev, const int key[10], int M, int Lmax, int precis
     GD_TRY(cudaMalloc(&c.d_state, sizeof(GdState)));
     GD_TRY(cudaMallocHost(&c.h_state, sizeof(GdState)));
     GD_TRY(cudaMalloc(&c.slots, c.slot_bytes * (size_t)(Lmax + 1)));
-    GD_TRY(cudaMemset(c.slots, 0, c.slot_bytes * (size_t)(Lmax + 1)));
+    GD_TRY(cudaMemsetAsync(c.slots, 0, c.slot_bytes * (size_t)(Lmax + 1), st));
     GD_TRY(cudaEventCreate(&c.ev0));
     GD_TRY(cudaEventCreate(&c.ev1));
     GD_TRY(cudaGraphCreate(&c.graph, 0));
@@ -612,7 +613,7 @@ int estimate_on_device(double eps, int M, int Lmin, int Lmax, uint64_t N0, const
     }
     if (!c) {
         c = new GdCache();
-        const int rc = gd_build(*c, dev, key, M, Lmax, precision, model, payoff);
+        const int rc = gd_build(*c, dev, key, M, Lmax, precision, model, payoff, st);
         if (rc) {
             c->release();
             delete c;

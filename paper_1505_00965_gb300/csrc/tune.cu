@@ -126,7 +126,7 @@ int mlmc_autotune(int M, int max_level, int precision, int payoff, void *stream,
         if (e1) cudaEventDestroy(e1);
     };
     cudaError_t e = cudaMalloc(&ws, ws_bytes);
-    if (e == cudaSuccess) e = cudaMemset(ws, 0, ws_bytes);
+    if (e == cudaSuccess) e = cudaMemsetAsync(ws, 0, ws_bytes, st);
     if (e == cudaSuccess) e = cudaMalloc(&d_sums, 4 * sizeof(double));
     if (e == cudaSuccess) e = cudaEventCreate(&e0);
     if (e == cudaSuccess) e = cudaEventCreate(&e1);
