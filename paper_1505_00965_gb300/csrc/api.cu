@@ -15,6 +15,7 @@
 
 #include "driver.h"
 #include "engine.h"
+#include "fx_drift.h"
 #include "host.h"
 #include "mlmc.h"
 #include "rng.cuh"
@@ -412,6 +413,7 @@ static void fill_fixed_point(LevelParams &p, const mlmc_model *m, int M)
     p.fx = 0;
     p.fx_a = p.fx_c2 = 0;
     p.fx_rh = p.fx_base = 0;
+    p.fx_rest = 0;
     p.fx_fixed = 0;
     if (m->kind != MLMC_MODEL_GBM) return;
     // on level 0 the one increment is added to 1 - K / S0 and not multiplied: more of the range is left
@@ -426,10 +428,14 @@ static void fill_fixed_point(LevelParams &p, const mlmc_model *m, int M)
     p.fx = 63 - e;
     p.fx_a = (uint64_t)std::nearbyint(std::ldexp(p.a, p.fx + 6));
     p.fx_c2 = (uint64_t)std::nearbyint(std::ldexp(c2, p.fx + 6));
-    p.fx_rh = (int64_t)std::nearbyint(std::ldexp(drift, p.fx));
+    const FxDrift fd = fx_drift(drift, p.fx);
+    p.fx_rh = fd.rh;
+    p.fx_rest = fd.rest;
     // payoffs in the same units: the excess 1 - K / S0 + (G - 1) and its difference must fit
     if (!mil && (level0 || (M == 4 && p.nf == 4)) && (most + std::fabs(1.0 - p.pay_k64) < 0.999 * (1 << e) || level0)) {
         p.fx_fixed = 1;
+        p.fx_rh += p.fx_rest >> 31;  // one block: the nearest unit
+        p.fx_rest = 0;
         p.fx_base = (int64_t)std::nearbyint(std::ldexp(1.0 - p.pay_k64, p.fx));
     }
 }

@@ -31,9 +31,11 @@ struct LevelParams {
     // FP64 payoff constants of the same options: disc S0 and K / S0
     double pay_dS0_64, pay_k64;
     // FP64 steps in fixed point (fx_steps): their unit is 2^-fx, 0 where they run in FP64; sigma sqrt(h)
-    // and sigma^2 h / 2 in units of 2^-(fx + 6), r h (Milstein: r h - sigma^2 h / 2) in units of 2^-fx
+    // and sigma^2 h / 2 in units of 2^-(fx + 6), the whole units of r h
+    // (Milstein: r h - sigma^2 h / 2) in 2^-fx
     uint64_t fx_a, fx_c2;
     int64_t fx_rh;
+    uint32_t fx_rest;  // the fraction of a unit that fx_rh lacks (fx_drift.h)
     int fx;
     // samples of one Philox block at most (level 0; M^l = 4 with M = 4) whose payoff is formed in the
     // same units: 1 - K / S0, and whether it fits

@@ -19,6 +19,7 @@
 #include <type_traits>
 
 #include "engine.h"
+#include "fx_drift.h"
 #include "normal64.cuh"
 #include "packed.cuh"
 #include "rng.cuh"
@@ -294,49 +295,54 @@ __device__ __forceinline__ void fx_steps(const LevelParams &p, uint32_t slo, uin
     int64_t zsum = 0;   // Milstein: sum of its normals
     int q = 0;
     const R a = step_a<R, MIL>(p), c2 = step_c2<R, MIL>(p), rHm = R(M * (p.rh - p.c2));
-    for (int j = j0; j < j1; ++j) {
-        const uint4 x = philox_of<RK>(p, make_uint4(p.ctr3, (uint32_t)j, shi, slo));
-        int64_t d[4], z[4];
-        if constexpr (MIL) {
-            fx_pair(x.x, x.y, u23, tab, z[0], z[1]);
-            fx_pair(x.z, x.w, u23, tab, z[2], z[3]);
+    uint32_t rest = fx_drift_sum(p.fx_rest, j0 / kDriftCalls);
+    for (int g = j0; g < j1; g += kDriftCalls) {
+        const int64_t rh = fx_drift_next(p.fx_rh, p.fx_rest, rest);
+        const int ge = min(g + kDriftCalls, j1);
+        for (int j = g; j < ge; ++j) {
+            const uint4 x = philox_of<RK>(p, make_uint4(p.ctr3, (uint32_t)j, shi, slo));
+            int64_t d[4], z[4];
+            if constexpr (MIL) {
+                fx_pair(x.x, x.y, u23, tab, z[0], z[1]);
+                fx_pair(x.z, x.w, u23, tab, z[2], z[3]);
 #pragma unroll
-            for (int k = 0; k < 4; ++k) d[k] = fx_increment_milstein(z[k], p.fx_a, p.fx_c2, p.fx_rh);
-        } else {
-            fx_increment_pair(x.x, x.y, u23, tab, p.fx_a, p.fx_rh, d[0], d[1]);
-            fx_increment_pair(x.z, x.w, u23, tab, p.fx_a, p.fx_rh, d[2], d[3]);
-        }
-        four(d[0], d[1], d[2], d[3], fS, fsum, fhi);
-        if constexpr (ANTI) {
-            if constexpr (MT == 4) four(d[3], d[2], d[1], d[0], aS, asum, ahi);
-            else four(d[1], d[0], d[3], d[2], aS, asum, ahi);
-        }
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            dsum += d[k];
-            if constexpr (MIL) zsum += z[k];
-            bool coarse_now;
-            if constexpr (MT != 0) {
-                coarse_now = (k + 1) % MT == 0;
+                for (int k = 0; k < 4; ++k) d[k] = fx_increment_milstein(z[k], p.fx_a, p.fx_c2, rh);
             } else {
-                coarse_now = ++q == M;
-                if (coarse_now) q = 0;
+                fx_increment_pair(x.x, x.y, u23, tab, p.fx_a, rh, d[0], d[1]);
+                fx_increment_pair(x.z, x.w, u23, tab, p.fx_a, rh, d[2], d[3]);
             }
-            if (coarse_now) {
-                R dc;
-                if constexpr (MIL) {
-                    const R zc = (R)zsum;
-                    dc = fma(fma(c2, zc, a), zc, rHm);
+            four(d[0], d[1], d[2], d[3], fS, fsum, fhi);
+            if constexpr (ANTI) {
+                if constexpr (MT == 4) four(d[3], d[2], d[1], d[0], aS, asum, ahi);
+                else four(d[1], d[0], d[3], d[2], aS, asum, ahi);
+            }
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                dsum += d[k];
+                if constexpr (MIL) zsum += z[k];
+                bool coarse_now;
+                if constexpr (MT != 0) {
+                    coarse_now = (k + 1) % MT == 0;
                 } else {
-                    dc = fx_to_double_signed(dsum, unit);
+                    coarse_now = ++q == M;
+                    if (coarse_now) q = 0;
                 }
-                cS = fma(cS, dc, cS);
-                if constexpr (PAY == kAsian) csum += cS;
-                if constexpr (PAY == kLookback) {
-                    chi = max_positive(chi, cS);
-                    if constexpr (COARSE_LO) clo = fmin(clo, cS);
+                if (coarse_now) {
+                    R dc;
+                    if constexpr (MIL) {
+                        const R zc = (R)zsum;
+                        dc = fma(fma(c2, zc, a), zc, rHm);
+                    } else {
+                        dc = fx_to_double_signed(dsum, unit);
+                    }
+                    cS = fma(cS, dc, cS);
+                    if constexpr (PAY == kAsian) csum += cS;
+                    if constexpr (PAY == kLookback) {
+                        chi = max_positive(chi, cS);
+                        if constexpr (COARSE_LO) clo = fmin(clo, cS);
+                    }
+                    dsum = zsum = 0;
                 }
-                dsum = zsum = 0;
             }
         }
     }
