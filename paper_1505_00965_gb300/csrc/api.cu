@@ -428,7 +428,7 @@ static void fill_fixed_point(LevelParams &p, const mlmc_model *m, int M)
     p.fx = 63 - e;
     p.fx_a = (uint64_t)std::nearbyint(std::ldexp(p.a, p.fx + 6));
     p.fx_c2 = (uint64_t)std::nearbyint(std::ldexp(c2, p.fx + 6));
-    const FxDrift fd = fx_drift(drift, p.fx);
+    const FxDrift fd = fx_drift(drift, p.fx, mil ? fx_dropped_mean(p.fx_c2) : 0.0);
     p.fx_rh = fd.rh;
     p.fx_rest = fd.rest;
     // payoffs in the same units: the excess 1 - K / S0 + (G - 1) and its difference must fit

@@ -19,10 +19,18 @@ struct FxDrift {
     int64_t rh;
     uint32_t rest;
 };
-inline FxDrift fx_drift(double drift, int u)
+// more: units that each step's other products drop on average (Milstein).
+inline FxDrift fx_drift(double drift, int u, double more = 0.0)
 {
-    const double x = std::ldexp(drift, u), r = std::floor(x);
-    return {(int64_t)r, (uint32_t)std::ldexp(x - r, 32)};
+    const double x = std::ldexp(drift, u), r = std::floor(x), rest = x - r + more;
+    return {(int64_t)r + (int64_t)std::floor(rest), (uint32_t)std::ldexp(rest - std::floor(rest), 32)};
+}
+// The mean of what fx_mul64(a, b) lacks of a b 2^-64 over a: half a unit for each cross product and a
+// quarter of the low words' product, with b's own words.
+inline double fx_dropped_mean(uint64_t b)
+{
+    const uint32_t lo = (uint32_t)b;
+    return (b >> 32 ? 0.5 : 0.0) + (lo ? 0.5 : 0.0) + std::ldexp((double)lo, -33);
 }
 // The sum ahead of group g (half a unit to begin with: a single group takes the nearest unit), and the
 // drift of the next group.
@@ -35,7 +43,7 @@ MLMC_HOST_DEVICE int64_t fx_drift_next(int64_t rh, uint32_t rest, uint32_t &sum)
     return rh;
 }
 // Philox calls of a group.  Euler--Maruyama: 256 steps, whose 2^-55 S does not see; what the fine steps
-// take, the coarse ones do too.
-constexpr int kDriftCalls = 64;
+// take, the coarse ones do too.  Milstein: single calls, since its coarse path has the FP64 drift.
+template <bool MILSTEIN> constexpr int kDriftCalls = MILSTEIN ? 1 : 64;
 
 }  // namespace mlmcgb

@@ -260,8 +260,10 @@ __device__ __forceinline__ uint4 philox_of(const LevelParams &p, uint4 c)
 // product (and the functional the sum or the largest of its G) in one FP64 multiply-add each, where
 // FP64 steps take two to four per step.  The FP64 pipe takes a warp instruction every 64 cycles per
 // scheduler, a 64-bit integer product 12 cycles of the multiplier.  Increments and products are
-// exact to 2^-62 or better where (1 + dmax)^4 < 2 and to 2^-56 at worst, without a bias, and S
-// rounds once per call where four FP64 steps round four times.  Coarse steps run in FP64 with the
+// exact to 2^-62 or better where (1 + dmax)^4 < 2 and to 2^-56 at worst; the products' errors and, beyond
+// the normals' own, the increments' have a mean below 0.05 units (the drift carries its remainder and
+// what Milstein's square drops, fx_drift.h), since a bias would add up over the steps.  S rounds once
+// per call where four FP64 steps round four times.  Coarse steps run in FP64 with the
 // exact sum of their fine d.  The caller checks p.fx, whose rule also keeps every factor positive;
 // no kGeoAsian (it needs every step's value).
 // Measured on the Asian call at level 5 (M = 4), 3.0e5 samples: 23.9 ms with the library's normals,
@@ -295,10 +297,11 @@ __device__ __forceinline__ void fx_steps(const LevelParams &p, uint32_t slo, uin
     int64_t zsum = 0;   // Milstein: sum of its normals
     int q = 0;
     const R a = step_a<R, MIL>(p), c2 = step_c2<R, MIL>(p), rHm = R(M * (p.rh - p.c2));
-    uint32_t rest = fx_drift_sum(p.fx_rest, j0 / kDriftCalls);
-    for (int g = j0; g < j1; g += kDriftCalls) {
+    constexpr int group = kDriftCalls<MIL != kEuler>;
+    uint32_t rest = fx_drift_sum(p.fx_rest, j0 / group);
+    for (int g = j0; g < j1; g += group) {
         const int64_t rh = fx_drift_next(p.fx_rh, p.fx_rest, rest);
-        const int ge = min(g + kDriftCalls, j1);
+        const int ge = min(g + group, j1);
         for (int j = g; j < ge; ++j) {
             const uint4 x = philox_of<RK>(p, make_uint4(p.ctr3, (uint32_t)j, shi, slo));
             int64_t d[4], z[4];

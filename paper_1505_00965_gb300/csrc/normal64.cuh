@@ -249,11 +249,14 @@ MLMC_FX void fx_increment_pair(uint32_t xa, uint32_t xb, bool u23, const uint64_
     d1 = rh + (int64_t)((fx_mul64(ra, fx_swapped(t) ? c : s) ^ m1) - m1);
 }
 // The Milstein increment r h - c2 + sigma sqrt(h) z + c2 z^2 from z in units of 2^-58; A and C2 in
-// units of 2^-(u + 6), rhm in units of 2^-u.
+// units of 2^-(u + 6), rhm in units of 2^-u.  |z| < 2^61 leaves room to square 8 z, so that z^2 keeps units of
+// 2^-58 (2^-52 from z itself: rms error 2^-51.4 where an FP64 product has 2^-52.3).  The product with A drops
+// as much for z as for -z; what the one with C2 drops is never negative, and the drift carries its mean
+// (fx_dropped_mean).
 MLMC_FX int64_t fx_increment_milstein(int64_t z, uint64_t A, uint64_t C2, int64_t rhm)
 {
-    const uint64_t m = (uint64_t)(z >> 63), y = ((uint64_t)z ^ m) - m;
-    return rhm + (int64_t)(((fx_mul64(y, A) ^ m) - m) + fx_mul64(fx_mul64(y, y) << 6, C2));
+    const uint64_t m = (uint64_t)(z >> 63), y = ((uint64_t)z ^ m) - m, y8 = y << 3;
+    return rhm + (int64_t)(((fx_mul64(y, A) ^ m) - m) + fx_mul64(fx_mul64(y8, y8), C2));
 }
 
 #ifdef __CUDACC__
