@@ -28,7 +28,7 @@ struct LevelParams {
     // FP32 payoff constants of the call options on paths relative to S0 (rel_payoff): disc S0,
     // -disc K, and for the fine (f) and coarse (c) path disc S0 / n, disc S0 / (2 n) - disc K
     float pay_dS0, pay_mdK, pay_af, pay_bf, pay_ac, pay_bc;
-    // FP64 payoff constants of the same options: disc S0 and K / S0
+    // FP64 constants of the payoffs formed in fixed point (fx_fixed): disc S0 and K / S0
     double pay_dS0_64, pay_k64;
     // FP64 steps in fixed point (fx_steps): their unit is 2^-fx, 0 where they run in FP64; sigma sqrt(h)
     // and sigma^2 h / 2 in units of 2^-(fx + 6), the whole units of r h

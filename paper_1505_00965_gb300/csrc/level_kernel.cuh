@@ -157,11 +157,12 @@ __device__ __forceinline__ float rel_payoff(const LevelParams &p, bool coarse, f
     else return fmaxf(fmaf(coarse ? p.pay_ac : p.pay_af, fmaf(-0.5f, S, sum), coarse ? p.pay_bc : p.pay_bf), 0.f);
 }
 
-// FP64 paths, the same options: the excess max(f - K / S0, 0) of the path's functional f relative to
-// S0, to be multiplied by disc S0 once per sample after the fine and coarse excesses are
-// subtracted.  The trapezoid average is (sum' - S_n' / 2) / n + 1 / (2 n), n a power of two, so the
-// fine and coarse path use exactly the same constants and no rounding of a constant enters their
-// difference.  4 to 8 FP64 operations per sample where payoff_from on the values times S0 took 9 to 19.
+// FP64 paths, the same options: the excess max(S0 f - K, 0) of the path's functional f relative to S0,
+// to be multiplied by disc once per sample after the fine and coarse excesses are subtracted.  The
+// trapezoid average is (sum' - S_n' / 2) / n + 1 / (2 n), n a power of two, so the fine and coarse path use
+// exactly the same constants and no rounding of a constant enters their difference.  S0 and K enter one
+// multiply-add as they are: K / S0 overflows and disc S0 underflows for options that the payoff itself
+// is finite for.  4 to 8 FP64 operations per sample where payoff_from on the values times S0 took 9 to 19.
 // fmax(x, 0) (0 for NaN) and, for hi >= 0 and x not NaN, fmax(hi, x), on the bit patterns: an FP64
 // comparison occupies the FP64 pipe as an FP64 addition does.
 __device__ __forceinline__ double positive_part(double x)
@@ -179,18 +180,18 @@ template <int PAY> __device__ __forceinline__ double rel_excess(const LevelParam
 {
     double f = PAY == kLookback ? hi : S;
     if constexpr (PAY == kAsian) f = fma(fma(-0.5, S, sum), inv_n, 0.5 * inv_n);
-    return positive_part(sub_rn(f, p.pay_k64));
+    return positive_part(fma(f, p.S0, -p.K));
 }
 template <typename R, int PAY, int MIL> __device__ __forceinline__ R path_scale(const LevelParams &p, R Y)
 {
-    if constexpr (kRelExcess<R, PAY> && MIL != kLibrary) return mul_rn(R(p.pay_dS0_64), Y);
+    if constexpr (kRelExcess<R, PAY> && MIL != kLibrary) return mul_rn(R(p.disc), Y);
     else return Y;
 }
 
 // Payoff of one whole path relative to S0 (values S, sum, hi, log-sum ls after its n steps, 1/n =
 // inv_n; `coarse` picks the coarse path): a relative form above where it exists, else
 // payoff_value on the values times S0.  Differences and means of payoffs go through path_scale,
-// which applies the FP64 forms' common factor disc S0.
+// which applies the FP64 forms' common factor disc.
 template <typename R, int PAY, int MIL>
 __device__ __forceinline__ R path_payoff(const LevelParams &p, bool coarse, R S, R sum, R hi, R ls, R S0, R logS0,
                                          R inv_n)
@@ -910,12 +911,12 @@ struct FixedMoments {
     }
     __device__ __forceinline__ void fold(const LevelParams &p, double m[4]) const
     {
-        const double w = p.pay_dS0_64, w2 = w * w;
+        const double w = p.pay_dS0_64;  // one factor at a time: w^4 may overflow where the sum does not
         const double top = (double)(int64_t)(s1 >> 32) * 4294967296.0 + (double)(uint32_t)s1;
         m[0] += w * ldexp(top, -p.fx);
-        m[1] += w2 * m2;
-        m[2] += w2 * w * m3;
-        m[3] += w2 * w2 * m4;
+        m[1] += w * (w * m2);
+        m[2] += w * (w * (w * m3));
+        m[3] += w * (w * (w * (w * m4)));
     }
 };
 __device__ __forceinline__ int64_t max0(int64_t x) { return x > 0 ? x : 0; }
@@ -1145,7 +1146,9 @@ __device__ __forceinline__ void block_increments(const LevelParams &p, uint32_t 
 // value as payoff_value on the one-step path in exact arithmetic: European disc (S_1 - K)^+;
 // arithmetic Asian (trapezoid, n = 1) A = (S_0 + S_1) / 2 = S_0 (1 + d / 2); lookback
 // max(S_0, S_1) = S_0 (1 + max(d, 0)).  The argument v is d on FP32 paths (d = r h + sigma dW) and the
-// normal z itself on FP64 paths, where the multiply-add that would form d costs as much as 64 FP32 ones.
+// normal z on FP64 paths (samples that fixed_level0 does not take: |1 - K / S0| above 14, or sigma sqrt(T)
+// above 2).  Scaling z to units of one first costs a multiply, but a slope in units of 2^-58 would
+// underflow for S0 below 1e-290.
 template <int PAY> constexpr bool kLevel0Affine = PAY == kEuropean || PAY == kAsian || PAY == kLookback;
 template <typename R> struct Level0Consts {
     R slope, at0, floor;  // payoff = max(slope v + at0, floor)
@@ -1155,7 +1158,7 @@ template <typename R, int PAY> __device__ __forceinline__ Level0Consts<R> level0
     const double w = p.disc * p.S0 * (PAY == kAsian ? 0.5 : 1.0), base = p.disc * (p.S0 - p.K);
     const R floor = PAY == kLookback ? fmax(R(base), R(0)) : R(0);
     if constexpr (sizeof(R) == 4) return {R(w), R(base), floor};
-    else return {w * step_a<R, kEuler>(p), fma(w, p.rh, base), floor};
+    else return {w * p.a, fma(w, p.rh, base), floor};
 }
 // Lookback: max(fma(max(d, 0), dS0, dS0mK), 0) = max(fma(d, dS0, dS0mK), max(dS0mK, 0)) exactly,
 // since dS0 > 0: for d > 0 the fma rounds to at least dS0mK, and for d <= 0 it rounds to at most
@@ -1186,7 +1189,7 @@ __device__ __forceinline__ void small_block(const LevelParams &p, uint64_t q, ui
 #pragma unroll
         for (int r = 0; r < 4; ++r) {
             if constexpr (kLevel0Affine<PAY> && !MIL) {
-                Y[r] = level0_payoff<R>(sizeof(R) == 8 ? z[r] : d[r], level0_consts<R, PAY>(p));
+                Y[r] = level0_payoff<R>(sizeof(R) == 8 ? z[r] * R(kFxZ) : d[r], level0_consts<R, PAY>(p));
             } else {
                 R fS = R(1), fsum = R(0), fhi = R(1), flo = R(1), fls = R(0);
                 em_step<R, PAY, false>(fS, fsum, fhi, flo, fls, d[r]);
@@ -1207,7 +1210,7 @@ __device__ __forceinline__ void small_block(const LevelParams &p, uint64_t q, ui
         R Y;
         if (nf == 1) {
             if constexpr (kLevel0Affine<PAY> && !MIL) {
-                Y = level0_payoff<R>(sizeof(R) == 8 ? z[r] : d[r], level0_consts<R, PAY>(p));
+                Y = level0_payoff<R>(sizeof(R) == 8 ? z[r] * R(kFxZ) : d[r], level0_consts<R, PAY>(p));
             } else {
                 em_step<R, PAY, false>(fS, fsum, fhi, flo, fls, d[r]);
                 Y = payoff_value<R, PAY>(S0 * fS, S0 * fsum, S0 * fhi, logS0 + fls, inv_nf, p);
@@ -1317,7 +1320,7 @@ __device__ __forceinline__ void small_range(const LevelParams &p, uint64_t first
 #pragma unroll
                 for (int r = 0; r < 4; ++r) {
                     if constexpr (kLevel0Affine<PAY> && !MIL) {
-                        Y[r] = level0_payoff<R>(sizeof(R) == 8 ? z[r] : d[r], c0);
+                        Y[r] = level0_payoff<R>(sizeof(R) == 8 ? z[r] * R(kFxZ) : d[r], c0);
                     } else {
                         R fS = R(1), fsum = R(0), fhi = R(1), flo = R(1), fls = R(0);
                         em_step<R, PAY, false>(fS, fsum, fhi, flo, fls, d[r]);
