@@ -596,8 +596,14 @@ int acquire_scratch(size_t ws_bytes, DriverScratch **out)
 
 void release_scratch(DriverScratch *s)
 {
-    std::lock_guard<std::mutex> lock(g_pool_mutex);
-    g_pool.push_back(s);
+    {
+        std::lock_guard<std::mutex> lock(g_pool_mutex);
+        if (s->ws_bytes <= kMaxPooledBytes && g_pool.size() < kMaxPooledSets) {
+            g_pool.push_back(s);
+            return;
+        }
+    }
+    free_scratch(s);
 }
 
 }  // namespace mlmcgb

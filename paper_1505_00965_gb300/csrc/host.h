@@ -79,6 +79,9 @@ constexpr int kDriverSumsPerLevel = 16;
 constexpr int kDriverStreams = 4;
 // Every set's workspace holds at least this much, so that the small calls and the drivers share sets.
 constexpr size_t kMinScratchBytes = size_t(1) << 20;
+// What the pool keeps between calls at most: sets whose workspace an explicit grid made larger, and sets of
+// more calls at a time than this, are freed when their call ends.
+constexpr size_t kMaxPooledBytes = size_t(16) << 20, kMaxPooledSets = 64;
 struct DriverScratch {
     int device = -1;
     void *ws = nullptr;
