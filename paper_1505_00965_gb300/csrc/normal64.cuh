@@ -23,9 +23,12 @@
 //            level 2, 1e7 samples: 0.902 -> 0.850 ms; Asian level 5, 3.0e5 samples: 1.759 -> 1.663 ms).
 //
 // Error (against quadruple precision, 3e6 random words and the edges of every reduction): cos and sin
-// 2^-61.2 rms and 2^-58.2 at most, rho 2^-58.7 rms, 2^-56.8 at most from rho = 1/2 on and 2^-53.7 at
-// most (next to u = 1, where rho itself is below 2^-4).  An FP64 normal of size 1 to 2 rounds by up to
-// 2^-53.
+// 2^-61.2 rms and 2^-58.2 at most, rho 2^-58.8 rms, 2^-56.8 at most from rho = 1/2 on and 2^-53.7 at
+// most (rho about 2^-4).  The library's log and sqrt give rho with 2^-53.6 rms; the fixed-point error is
+// absolute where theirs shrinks with rho: below rho = 0.2 (one word in 64) it is 2^-55.6 to 2^-57.1 rms by
+// octave of 1 - u against 2^-56.7 to 2^-58.6, next to u = 1 (1 - u < 2^-10) 2^-56.2 against 2^-59.0
+// (2^-59.2 with the cubic term in 64 bits there: 1.1 % more time, no digit of a sum).  An
+// FP64 normal of size 1 to 2 rounds by up to 2^-53.
 #pragma once
 #include <cstdint>
 #ifndef __CUDACC__
