@@ -873,8 +873,8 @@ extern "C" int mlmc_estimate(double eps, int M, int Lmin, int Lmax, uint64_t N0,
         free_scratch(sc);
         return fail(MLMC_ECUDA, "%s failed: %s", what, cudaGetErrorString(e));
     };
-    // the completion tickets are zero after every finished launch; clear them in case an earlier
-    // call on this set stopped between a launch and its completion
+    // only the first slot's ticket is zero in a pooled set: a call of one slot (level sums, network gradients)
+    // may have written where the others lie
     cudaError_t e = rs.clear_tickets(kTicketBytes);
     if (e != cudaSuccess) return cuda_fail(e, "cudaMemsetAsync");
 

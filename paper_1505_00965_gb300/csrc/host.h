@@ -69,8 +69,9 @@ struct TunedShape {
 bool tuned_lookup(int precision, int payoff, int M, int level, uint64_t N, TunedShape *out);
 
 // Buffers of one call with host results (adaptive drivers, level sums, control variate), pooled per
-// device between calls: a workspace of at least ws_bytes (every slot's ticket zero in a set that is
-// in the pool), device and pinned host sums (kDriverSumsPerLevel doubles per level),
+// device between calls: a workspace of at least ws_bytes (its first ticket is zero in a set that is in the
+// pool; the calls of one slot write what they like behind it, so callers of several slots clear
+// theirs, RoundStreams::clear_tickets), device and pinned host sums (kDriverSumsPerLevel doubles per level),
 // two timing events, and kDriverStreams - 1 streams with their fork and join events, over which
 // (with the caller's stream) a round spreads its level launches.  acquire_scratch takes a set
 // from the pool or makes one; release_scratch returns it; free_scratch destroys a set that met

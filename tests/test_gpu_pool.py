@@ -1,4 +1,4 @@
-"""The pool of call buffers between calls: bounded."""
+"""The pool of call buffers between calls: bounded, and a set serves any call after any other."""
 import numpy as np
 import pytest
 
@@ -28,3 +28,23 @@ def test_a_large_grids_workspace_is_given_back(mlmc):
     for blocks in (1 << 21, 3 << 20):  # 64 and 96 MiB of block sums
         assert np.allclose(call(blocks), want, rtol=1e-5, atol=1e-3)
     assert torch.cuda.mem_get_info()[0] > free - (32 << 20)
+
+
+def test_estimate_after_a_gradient_on_the_same_buffers(mlmc):
+    """The gradient's parameters and outputs lie over the later slots' tickets of the driver's workspace."""
+    import torch
+
+    rng = np.random.default_rng(5)
+    theta = (0.2 * rng.standard_normal(mlmc.MLMC_CV_PARAMS)).astype(np.float32)
+    X = torch.tensor(rng.standard_normal((65536, 16)).astype(np.float32), device="cuda")
+    Y = torch.tensor(rng.standard_normal(65536).astype(np.float32), device="cuda")
+    before = mlmc.mlmc_set_driver_mode("host")
+    try:
+        mlmc.mlmc_shutdown()
+        want = mlmc.mlmc_estimate(1e-2, mlmc.Problem(payoff="asian"), 3).sums
+        mlmc.mlmc_shutdown()
+        mlmc.mlmc_mlp_grad(theta, X, Y, 65536)
+        got = mlmc.mlmc_estimate(1e-2, mlmc.Problem(payoff="asian"), 3).sums
+    finally:
+        mlmc.mlmc_set_driver_mode(before)
+    assert np.array_equal(np.asarray(got), np.asarray(want))
