@@ -118,6 +118,8 @@ enum { MLMC_TAG_PATHS = 0, MLMC_TAG_CV_MEAN = 1, MLMC_TAG_CV_TRAIN = 2 };
 
 /* Launch shape of one level kernel.  Zero in a field means "choose automatically".
  *   threads_per_block  multiple of 32, 32..1024 (at most 512 with samples_per_thread = 2)
+ *                      FP64 kernels hold 37 KB of tables per block, so an SM takes six blocks of any
+ *                      size: 32 or 64 threads leave most of it empty
  *   lanes_per_path     1 (one thread per sample) or a power of two up to 32: that many lanes of
  *                      one warp split the time steps of one sample into equal chunks and join
  *                      them by a product scan (GBM's step is multiplicative); requires
@@ -130,15 +132,17 @@ typedef struct mlmc_launch {
     int32_t lanes_per_path;
     int32_t blocks;
     int32_t samples_per_thread;  /* 1 or 2 (0 = automatic): with 2, each thread of a one-thread-
-                              per-sample launch steps two samples' paths in lockstep (two
-                              independent Philox and step chains for the scheduler to interleave);
-                              FP32 Euler--Maruyama paths of the coupled or single-level estimator
-                              with M^l >= 4 and lanes_per_path = 1 only.  Thread t of a grid of
-                              T threads takes samples t, t + T, ... as with 1, in pairs, and runs
-                              an unpaired last sample alone; the automatic grid is the same.  The
-                              samples and their Y are the same; the FP32 moment sums add them in
-                              another order.  Automatic: 2 for FP32 Euler--Maruyama whole paths
-                              with M = 4 and M^l >= 4, else 1 (or the autotuner's choice). */
+                              per-sample launch steps two samples' paths in lockstep, on packed
+                              pairs; FP32 Euler--Maruyama paths of the coupled or single-level
+                              estimator with M^l >= 4 and lanes_per_path = 1 only.  Thread t of a
+                              grid of T threads takes samples t, t + T, ... as with 1, in pairs,
+                              and runs an unpaired last sample alone; the automatic grid is the
+                              same, and on one grid so are the samples, their Y and the sums.
+                              Automatic (unless the autotuner chose): pairs for FP32 whole paths
+                              with M = 4 and M^l >= 4, of either scheme and every estimator, and
+                              for a few long FP32 paths one sample per lane group in blocks whose
+                              other warps form the increments.  An explicit 1 takes the plain
+                              one-sample kernel in each of these cases. */
 } mlmc_launch;
 
 /* Message describing the last failure on this host thread ("" if none). */

@@ -228,7 +228,6 @@ int plan_level(int level, int M, uint64_t N, int precision, int payoff, int sche
     plan->threads = threads;
     plan->lanes = lanes;
     plan->blocks = blocks;
-    plan->ns = ns;
     return MLMC_OK;
 }
 
@@ -333,7 +332,6 @@ static int plan_idle(int level, int M, uint64_t N, int precision, const mlmc_mod
                 plan->kernel = k;
                 plan->threads = relay;
                 plan->blocks = (int)lane_warps;
-                plan->ns = 1;
             }
         }
     }

@@ -32,7 +32,6 @@ int max_resident_blocks(const void *kernel, int threads, int *out);
 struct Plan {
     const void *kernel;
     int threads, lanes, blocks;
-    int ns = 1;  // samples per thread (2: the two-sample kernel)
 };
 int plan_level(int level, int M, uint64_t N, int precision, int payoff, int scheme, const mlmc_launch *launch,
                Plan *plan);
