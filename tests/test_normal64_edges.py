@@ -29,6 +29,10 @@ extern "C" void words(const uint32_t *x, long n, int u23, uint32_t *w)
 {
     for (long i = 0; i < n; ++i) w[i] = fx_word(x[i], u23 != 0);
 }
+extern "C" void doubles(const uint64_t *x, long n, int unit, uint64_t *d)
+{
+    for (long i = 0; i < n; ++i) d[i] = fx_double_bits<true>(x[i], unit);
+}
 """
 L = np.longdouble
 
@@ -93,3 +97,12 @@ def test_table_entries():
         assert have == ln2 + lnc + cos + [0]
         two_pi = re.search(r"kFxTwoPi60 = 0x([0-9A-F]+)", text).group(1)
         assert int(two_pi, 16) == int(mp.nint(2 * mp.pi * 2 ** 60))
+
+
+def test_conversion_rounds_to_nearest(lib):
+    rng = np.random.default_rng(6)
+    x = (rng.integers(1, 1 << 63, 50_000) >> rng.integers(0, 60, 50_000)).astype(np.uint64)
+    d = np.zeros(len(x), np.uint64)
+    lib.doubles(x.ctypes.data_as(ctypes.c_void_p), ctypes.c_long(len(x)), 60, d.ctypes.data_as(ctypes.c_void_p))
+    want = x.astype(L) * L(2) ** -60  # 64-bit mantissa: exact
+    assert np.all(np.abs(d.view(np.float64).astype(L) - want) <= want * L(2) ** -53)
