@@ -132,7 +132,7 @@ def _oracle_job(args):
 # DRAM bytes (read + write) of one launch of the dominant kernel, from ncu (level_ns2_kernel, lookback,
 # level 6, N = 10^6, two samples per thread): the kernels read no input arrays; the algorithmic
 # bytes are the block partials and the four sums (608 x 32 + 32 = 19.5 KB).
-TRAFFIC_BYTES_PER_LAUNCH = 97280
+TRAFFIC_BYTES_PER_LAUNCH = 78336
 TRAFFIC_BASIS = ("ncu dram__bytes_read.sum + dram__bytes_write.sum of one level_ns2_kernel launch (lookback, "
                  "level 6, N=1e6, 608 blocks); algorithmic bytes 19.5 KB of block partials")
 # Widening 32-bit integer products per coupled step of the FP64 paths (normals and step products are
@@ -456,6 +456,8 @@ def gpu_arm(args) -> None:
     peak = sms * SCHEDULERS_PER_SM * WARP * max_mhz * 1e6 / 1e9          # G instructions / s
     achieved = instr / (kern_ms / 1e3) / 1e9
     roofline = {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "Ginstr/s", "frac": achieved / peak,
+                "frac_basis": "algorithmic instructions of the scalar form (level_instructions) over the issue peak; "
+                              "packed FP32x2 operations do two in one, so fewer issue slots are busy",
                 "traffic": TRAFFIC_BYTES_PER_LAUNCH, "traffic_basis": TRAFFIC_BASIS,
                 "kernel": "level_ns2_kernel, level_kernel and level_small_kernel (FP32 paths, all levels of the "
                           "step; time = the driver's events around each "

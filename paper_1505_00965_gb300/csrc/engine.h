@@ -91,9 +91,12 @@ const void *level_anti_kernel_fp64_library(int payoff, int mt, bool long_lanes);
 // round alike.  Against that form, over 57 cases each of 1e5 to 2.5e8 steps, S0 = K = 100, r = 0.05,
 // sigma = 0.2, the largest difference of the four sums with fixed-point normals and steps was 2.4e-11 on
 // M = 4 level 5, 7e-11 on M = 2 level 10, 6e-10 on level 11 (9 cases above 1e-10), 2.2e-9 and 4.4e-9 at 4096
-// steps and 2e-7 at 65536 (with fixed-point normals alone 8e-9 there); the strong order 1/2 of
-// Euler--Maruyama, coupled or antithetic, keeps all of its levels below 8e-10.  The single-level
-// estimator has no such difference.
+// steps and 2e-7 at 65536 (with fixed-point normals alone 8e-9 there).  It costs 24.9 ms for 3e8 steps where
+// fixed point took 1.7.  Euler--Maruyama, of strong order 1/2, keeps fixed point: over 3000 drawn launches
+// of every kind three differed by more than 1e-9 (in the norm of the four sums), of 9, 10 and 39 samples at
+// 65536 steps whose Y nearly cancel; against extended precision the fixed-point sums were the nearer ones
+// there (4.8e-10, 8.2e-10, 1.1e-10 against 2.0e-9, 1.2e-9, 1.8e-9).  The single-level estimator has no
+// such difference.
 constexpr long kMilsteinFixedSteps = 1024;
 inline int path_scheme(bool fp64, int scheme, bool single_level, long nf)
 {
@@ -150,7 +153,8 @@ __host__ __device__ inline double lane_waves(double w, bool fp64)
     const double part = fp64 ? 0.2 + 0.95 * w : 3.0 * w, least = fp64 ? 0.26 : 0.25;
     return part < least ? least : part < 1.0 ? part : 1.0;
 }
-// FP64: 1000 samples of level 3 take 16.5 us on lanes of 32 steps, 12.4 of 8; level 4 18.5 and 14.4.
+// FP64, 1000 samples: level 3 takes 19.4 us on lanes of 32 steps, 15.3 of 16 and 14.4 of 8; level 4 20.5, 16.5
+// and 18.5 (128 threads per block).
 __host__ __device__ constexpr long min_lane_steps(bool fp64) { return fp64 ? 8 : 256; }
 // The control variate's level-estimator kernel (cv_level.cu) for a payoff on level `level` with
 // refinement M: compiled for M^l = 1, 4, 16 at M = 4, else for a run-time M^l; NULL for an unknown

@@ -1557,8 +1557,8 @@ __global__ void __launch_bounds__(1024) level_small_kernel(const LevelParams p)
 // ------------------------------------------------------------------ batched rounds
 
 // Samples per thread of the batched kernel's whole paths: FP32 pairs (simulate_pair), the same samples
-// in the same order per thread.  The 96-problem batch: 357 -> 348 ms; three blocks per SM (80
-// registers) 352 ms.
+// in the same order per thread.  Books of fewer and of 96 problems: 54.9 -> 53.8 ms, 13.36 -> 12.97, 357 -> 348;
+// three blocks per SM (80 registers) 352 ms on the last.
 template <typename R> constexpr int kBatchSamples = sizeof(R) == 4 ? 2 : 1;
 // All samples of one chunk, by the threads of one block, on the code path of the chunk's task.
 // Y of sample first + i goes to y[i] when the task has per-sample output (p.y_out, indexed from

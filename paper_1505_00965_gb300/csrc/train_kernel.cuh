@@ -302,7 +302,7 @@ __device__ __forceinline__ void train_contract(const TrainSmem &s, int nrows, fl
 // Training (TRAIN) of the networks of a.job[cluster index], or one gradient evaluation (!TRAIN) of
 // a.job[0]'s network on one batch shared by every cluster of the launch.  A gradient of 65536 rows on
 // one cluster of 16 CTAs left 136 SMs idle for 16 chunks of rows: the whole call took 264 us, 75 us on
-// eight clusters with the loss formed on the device.
+// the seven clusters that the GPU holds at once (112 CTAs of three chunks), with the loss formed on the device.
 template <bool TRAIN>
 __global__ void __launch_bounds__(kTrainThreads, 1) train_cluster_kernel(const TrainArgs a)
 {
