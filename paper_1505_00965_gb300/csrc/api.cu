@@ -308,7 +308,7 @@ static int plan_idle(int level, int M, uint64_t N, int precision, const mlmc_mod
         if (precision == MLMC_FP32_PATH) {
             while (plan->threads > 64 && plan->threads % 64 == 0 && std::ceil(items / plan->threads) < sms) plan->threads /= 2;
             if (plan->threads < 256) plan->blocks = std::max(1, (int)std::ceil(items / plan->threads));
-        } else if (path_scheme(true, model->scheme, payoff->estimator == MLMC_SINGLE_LEVEL, nf) != kLibrary) {
+        } else if (path_scheme(true, model->scheme, payoff->estimator == MLMC_SINGLE_LEVEL, nf, N) != kLibrary) {
             constexpr int kThreads = 128;
             int resident = 0;
             if ((rc = max_resident_blocks(plan->kernel, kThreads, &resident))) return rc;
@@ -342,7 +342,7 @@ int plan_problem(int level, int M, uint64_t N, int precision, const mlmc_model *
                  const mlmc_launch *launch, Plan *plan, bool spread)
 {
     const int scheme = path_scheme(precision != MLMC_FP32_PATH, model->scheme,
-                                   payoff->estimator == MLMC_SINGLE_LEVEL, ipow(M, level));
+                                   payoff->estimator == MLMC_SINGLE_LEVEL, ipow(M, level), spread ? N : kManySamples);
     if (model->kind == MLMC_MODEL_QUINTIC_ODE) return plan_ode(level, M, N, precision, model->scheme, launch, plan);
     if (payoff->estimator != MLMC_ANTITHETIC) {
         const int rc = plan_level(level, M, N, precision, payoff->kind, scheme, launch, plan);

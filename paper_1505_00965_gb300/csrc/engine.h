@@ -85,22 +85,32 @@ const void *level_kernel_fp64_milstein(int payoff, int mt, bool split, bool long
 // The same kernels with FP64 steps on the CUDA library's normals (level_fp64_library.cu).
 const void *level_kernel_fp64_library(int payoff, int mt, bool split, bool long_lanes, bool positive);
 const void *level_anti_kernel_fp64_library(int payoff, int mt, bool long_lanes);
-// FP64 Milstein paths of more than 1024 fine steps take the library's logarithm, root and sine, and FP64
-// steps, operation for operation.  P_l - P_{l-1} of strong order 1 shrinks like 1 / n while the rounding
-// of its two paths grows like sqrt(n): at 4096 steps a level's sums agree to 1e-9 only between forms that
-// round alike.  Against that form, over 57 cases each of 1e5 to 2.5e8 steps, S0 = K = 100, r = 0.05,
-// sigma = 0.2, the largest difference of the four sums with fixed-point normals and steps was 2.4e-11 on
-// M = 4 level 5, 7e-11 on M = 2 level 10, 6e-10 on level 11 (9 cases above 1e-10), 2.2e-9 and 4.4e-9 at 4096
-// steps and 2e-7 at 65536 (with fixed-point normals alone 8e-9 there).  It costs 24.9 ms for 3e8 steps where
-// fixed point took 1.7.  Euler--Maruyama, of strong order 1/2, keeps fixed point: over 3000 drawn launches
-// of every kind three differed by more than 1e-9 (in the norm of the four sums), of 9, 10 and 39 samples at
-// 65536 steps whose Y nearly cancel; against extended precision the fixed-point sums were the nearer ones
-// there (4.8e-10, 8.2e-10, 1.1e-10 against 2.0e-9, 1.2e-9, 1.8e-9).  The single-level estimator has no
-// such difference.
-constexpr long kMilsteinFixedSteps = 1024;
-inline int path_scheme(bool fp64, int scheme, bool single_level, long nf)
+// Level sums of FP64 Milstein paths of more than 1024 fine steps over fewer than 4096 samples (of more
+// than 512 over fewer than 64) take the library's logarithm, root and sine, and FP64 steps, operation for
+// operation.  P_l - P_{l-1} of strong order 1 shrinks like 1 / n while the rounding of its two paths grows
+// like sqrt(n), so few samples' sums agree to 1e-9 only between forms that round alike; over N samples the
+// difference falls like 1 / sqrt(N).  Largest
+// difference of fixed-point sums to the library's (norm of the four sums, 2640 launches of 1e4 to 3e8 steps, coupled
+// and antithetic, S0 = K = 100, r = 0.05, sigma = 0.2) by fine steps, M and samples below 64 / 512 / 4096 / above:
+//    1024 (2)  1.1e-9  1.4e-10  8.8e-11  1.5e-11     4096 (4)   2.0e-9  3.3e-10  1.5e-10  4.4e-11
+//    2048 (2)  4.4e-9  5.1e-10  8.9e-11  3.6e-11    16384 (4)   7.0e-8  1.7e-8   5.3e-10  1.8e-10
+//    8192 (2)  4.6e-8  5.3e-9   5.7e-10  2.6e-10    65536 (4)   3.9e-7  3.7e-8   1.7e-8   4.5e-10 (3 launches)
+// Beyond 16384 steps the least number of samples grows with n^3, which keeps n^1.5 / sqrt(N).  The library's
+// form takes 24.9 ms for 3e8 steps, fixed point 1.7.  The adaptive drivers (many) keep fixed point: their sums
+// build up over rounds, and no result of theirs divides by a deep level's sum alone.  Euler--Maruyama, of
+// strong order 1/2, keeps fixed point too: over 3000 drawn launches of every kind three differed by more than
+// 1e-9, of 9, 10 and 39 samples at 65536 steps whose Y nearly cancel; against extended precision the
+// fixed-point sums were the nearer ones there (4.8e-10, 8.2e-10, 1.1e-10 against 2.0e-9, 1.2e-9, 1.8e-9).  The
+// single-level estimator has no such difference.
+constexpr long kMilsteinFixedSteps = 512, kMilsteinFewSteps = 1024, kMilsteinCubeSteps = 16384;
+constexpr double kMilsteinFewSamples = 64.0, kMilsteinFixedSamples = 4096.0;
+constexpr uint64_t kManySamples = UINT64_MAX;
+inline int path_scheme(bool fp64, int scheme, bool single_level, long nf, uint64_t N)
 {
-    return fp64 && scheme == kMilstein && !single_level && nf > kMilsteinFixedSteps ? kLibrary : scheme;
+    if (!fp64 || scheme != kMilstein || single_level || nf <= kMilsteinFixedSteps) return scheme;
+    if (nf <= kMilsteinFewSteps) return (double)N < kMilsteinFewSamples ? kLibrary : scheme;
+    const double over = nf > kMilsteinCubeSteps ? (double)nf / kMilsteinCubeSteps : 1.0;
+    return (double)N < kMilsteinFixedSamples * over * over * over ? kLibrary : scheme;
 }
 // Antithetic level kernels (level_anti_fp32.cu, level_anti_fp64.cu): mt = 4 (M = 4) or 0 (M = 2).
 const void *level_anti_kernel_fp32(int payoff, int mt, int scheme, bool long_lanes);

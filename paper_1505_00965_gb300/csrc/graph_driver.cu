@@ -56,7 +56,6 @@ struct GdState {
     int small_levels;   // levels l < small_levels have M^l < 4 (4 / M^l samples per Philox block)
     int antithetic;     // one thread per sample, no split
     int fp64;           // FP64 paths (the lanes model's second fit)
-    int library_from;   // first level whose FP64 paths are the library's (path_scheme; the first fit)
     int ws_blocks;      // grid cap: blocks of a level's workspace slot
     uint64_t N0;
     int res1[MLMC_MAX_LEVELS], resp[MLMC_MAX_LEVELS];  // residencies the lanes model compares
@@ -159,7 +158,7 @@ __device__ void gd_plan(const GdState &s, int l, uint64_t dN, int &variant, int 
         need = ceil((ceil(Nd * (double)nf / 4.0) + 1.0) / threads);
     } else {
         if (nf >= 8 && !s.antithetic) {
-            const bool fp64 = s.fp64 != 0 && l < s.library_from;
+            const bool fp64 = s.fp64 != 0;
             double best = 0.0;
             for (int P = 1; P <= 32; P *= 2) {
                 if (P > 1 && (nf % P != 0 || (nf / P) % unit != 0 || nf / P < min_lane_steps(fp64))) break;
@@ -406,7 +405,8 @@ int level_kernels(int l, int M, int precision, const mlmc_model *model, const ml
     *out = LevelKernels{};
     const long nf = ipow(M, l);
     const int pay = payoff->kind;
-    const int scheme = path_scheme(precision != MLMC_FP32_PATH, model->scheme, payoff->estimator == MLMC_SINGLE_LEVEL, nf);
+    const int scheme = path_scheme(precision != MLMC_FP32_PATH, model->scheme, payoff->estimator == MLMC_SINGLE_LEVEL, nf,
+                                   kManySamples);
     const bool anti = payoff->estimator == MLMC_ANTITHETIC;
     auto pick = [&](int mt, bool split, bool long_lanes, bool positive) {
         return precision == MLMC_FP32_PATH ? level_kernel_fp32(pay, mt, split, scheme, long_lanes, positive)
@@ -642,9 +642,6 @@ int estimate_on_device(double eps, int M, int Lmin, int Lmax, uint64_t N0, const
     h.small_levels = small;
     h.antithetic = payoff->estimator == MLMC_ANTITHETIC ? 1 : 0;
     h.fp64 = precision != MLMC_FP32_PATH ? 1 : 0;
-    while (h.library_from <= Lmax &&
-           path_scheme(h.fp64 != 0, model->scheme, payoff->estimator == MLMC_SINGLE_LEVEL, ipow(M, h.library_from)) != kLibrary)
-        ++h.library_from;
     h.ws_blocks = c->ws_blocks;
     AdaptiveMLMC costs(eps, M, Lmin, Lmax, N0);  // C_l with the estimator's cost scale
     if (h.antithetic)

@@ -48,7 +48,8 @@ int estimate_on_device(double eps, int M, int Lmin, int Lmax, uint64_t N0, const
                        std::chrono::steady_clock::time_point t_start);
 void graph_driver_release(int dev);
 // spread: whether launches that leave SMs idle may take smaller blocks (the adaptive driver keeps 256
-// threads, the shape of its device rounds, whose sums its own repeat bit for bit).
+// threads, the shape of its device rounds, whose sums its own repeat bit for bit), and whether few
+// samples of a deep FP64 Milstein level take the library's form (path_scheme).
 int plan_problem(int level, int M, uint64_t N, int precision, const mlmc_model *model, const mlmc_payoff *payoff,
                  const mlmc_launch *launch, Plan *plan, bool spread = true);
 void fill_params(LevelParams &p, int level, int M, uint64_t N, uint64_t first,
